@@ -49,9 +49,7 @@
 //    on the rounded totals.
 //  * the tile shape (TY, TZ) is a template parameter; the batch autotuner
 //    times the candidates on the actual lattices and keeps the fastest.
-#include <cuda.h>
 #include <cuda_runtime.h>
-#include <cudaTypedefs.h>
 #include <stdlib.h>
 
 #include <algorithm>
@@ -61,8 +59,10 @@
 
 #include <vector>
 
+#include "packed_f32.cuh"
 #include "skyrme_device.cuh"
 #include "skyrme_internal.h"
+#include "tma.cuh"
 
 namespace skyrme {
 
@@ -75,7 +75,6 @@ template <int TY, int TZ, bool SEX = false> constexpr int nslot()
 {
     return TY * TZ >= 512 && !SEX ? 8 : 4;
 }
-constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s per plane copy
 
 // One lattice of a step launch: a kernel parameter for a single lattice, an
 // entry of a device table for a batch.
@@ -172,77 +171,6 @@ __host__ __device__ __forceinline__ void lock_run(const CtaSplit &sp, int b, int
     len = len < o1 - o ? len : o1 - o;
 }
 
-// ------------------------------------------------------------- PTX helpers
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p)
-{
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void mbar_init(unsigned long long *bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count)
-                 : "memory");
-}
-__device__ __forceinline__ void mbar_fence_init()
-{
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long *bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-                 "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(unsigned long long *bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ unsigned long long global_ns()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-    return t;
-}
-// Bounded wait: false when the phase did not complete within limit_ns.
-__device__ __forceinline__ bool mbar_wait(unsigned long long *bar, uint32_t parity,
-                                          unsigned long long limit_ns = kWaitLimitNs)
-{
-    if (mbar_try_wait(bar, parity)) return true;
-    const unsigned long long t0 = global_ns();
-    while (global_ns() - t0 < limit_ns)
-        if (mbar_try_wait(bar, parity)) return true;
-    return false;
-}
-// The same wait that also gives up once *flag is set (another warp's wait
-// failed); the flag is read only when the phase is not complete at once.
-__device__ __forceinline__ bool mbar_wait_flag(unsigned long long *bar, uint32_t parity,
-                                               const volatile int *flag)
-{
-    if (mbar_try_wait(bar, parity)) return true;
-    const unsigned long long t0 = global_ns();
-    while (*flag == 0 && global_ns() - t0 < kWaitLimitNs)
-        if (mbar_try_wait(bar, parity)) return true;
-    return false;
-}
-__device__ __forceinline__ void tma_plane(void *dst, const CUtensorMap *map,
-                                          unsigned long long *bar, int c0, int c1, int c2)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar))
-        : "memory");
-}
-
-
 // ------------------------------------------------- tensor memory helpers
 // Tensor memory (256 KiB per SM: 128 lanes x 512 columns of 32 bits) holds
 // each thread's ring of in-plane records.  Warp 0 allocates the CTA's
@@ -312,111 +240,6 @@ __device__ __forceinline__ void tmem_wait_ld12(float (&v)[12])
     asm volatile("tcgen05.wait::ld.sync.aligned;" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]), "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]) : : "memory");
 }
 
-// ------------------------------------------------- packed 4-vector helpers
-struct P4 {
-    float2 a, b;  // components (0,1) and (2,3)
-};
-__device__ __forceinline__ float2 bc(float s) { return make_float2(s, s); }
-__device__ __forceinline__ P4 ld4(const float4 &v) { return {make_float2(v.x, v.y), make_float2(v.z, v.w)}; }
-__device__ __forceinline__ float4 st4(const P4 &v) { return make_float4(v.a.x, v.a.y, v.b.x, v.b.y); }
-__device__ __forceinline__ P4 add(const P4 &u, const P4 &v) { return {__fadd2_rn(u.a, v.a), __fadd2_rn(u.b, v.b)}; }
-// u - v
-__device__ __forceinline__ P4 sub(const P4 &u, const P4 &v)
-{
-    return {__ffma2_rn(v.a, bc(-1.f), u.a), __ffma2_rn(v.b, bc(-1.f), u.b)};
-}
-__device__ __forceinline__ P4 mul(float2 s, const P4 &v) { return {__fmul2_rn(s, v.a), __fmul2_rn(s, v.b)}; }
-__device__ __forceinline__ P4 fma(float2 s, const P4 &v, const P4 &c)
-{
-    return {__ffma2_rn(s, v.a, c.a), __ffma2_rn(s, v.b, c.b)};
-}
-__device__ __forceinline__ float2 dot2(const P4 &u, const P4 &v, float2 acc)
-{
-    return __ffma2_rn(u.b, v.b, __ffma2_rn(u.a, v.a, acc));
-}
-__device__ __forceinline__ float hsum(float2 t) { return t.x + t.y; }
-__device__ __forceinline__ float dot(const P4 &u, const P4 &v)
-{
-    return hsum(__ffma2_rn(u.b, v.b, __fmul2_rn(u.a, v.a)));
-}
-// The unscaled stencils' weights, the same for every lattice (compile-time
-// constants: the compiler takes them from its constant bank instead of
-// registers, which matters in the batched kernels, whose lattice
-// descriptors live in global memory)
-__device__ __forceinline__ float2 kW8() { return make_float2(8.f, 8.f); }
-__device__ __forceinline__ float2 kWm16() { return make_float2(-16.f, -16.f); }
-__device__ __forceinline__ float2 kW30() { return make_float2(30.f, 30.f); }
-__device__ __forceinline__ float2 kXm1() { return make_float2(-2.f / 3.f, -2.f / 3.f); }
-__device__ __forceinline__ float2 kXm2() { return make_float2(1.f / 12.f, 1.f / 12.f); }
-
-// weighted first difference c1 (p1 - m1) + c2 (p2 - m2) (the mixed second
-// derivatives, of the u_i)
-__device__ __forceinline__ P4 fd1(const P4 &m2, const P4 &m1, const P4 &p1, const P4 &p2, float2 c1,
-                                  float2 c2)
-{
-    return fma(c2, sub(p2, m2), mul(c1, sub(p1, m1)));
-}
-// 12h d phi = 8 (p1 - m1) - (p2 - m2), w8 = (8, 8)
-__device__ __forceinline__ P4 fd1u(const P4 &m2, const P4 &m1, const P4 &p1, const P4 &p2,
-                                   float2 w8)
-{
-    return fma(w8, sub(p1, m1), sub(m2, p2));
-}
-// -12h^2 d^2 phi = (p2 + m2) + 30 c - 16 (p1 + m1), wm16 = (-16, -16), w30 = (30, 30)
-__device__ __forceinline__ P4 fd2n(const P4 &m2, const P4 &m1, const P4 &c, const P4 &p1,
-                                   const P4 &p2, float2 wm16, float2 w30)
-{
-    return fma(wm16, add(p1, m1), fma(w30, c, add(p2, m2)));
-}
-
-// ------------------------------------------------- double-float sums
-// The streaming kernel keeps its energy, charge and force sums as unevaluated
-// sums hi + lo of two floats (|lo| <= ulp(hi)/2), combined with the error-free
-// two-sum and FMA two-product transformations (Knuth, Dekker): about 48
-// significant bits on the FP32 pipe.  GB300's FP64 pipe issues 2 operations
-// per SM and cycle, so FP64 reductions at the end of a launch sit on the
-// critical path; these do not.
-struct DF {
-    float hi, lo;
-};
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
-{
-    s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-__device__ __forceinline__ DF quick_two_sum(float a, float b)  // |a| >= |b|
-{
-    const float s = __fadd_rn(a, b);
-    return {s, __fsub_rn(b, __fsub_rn(s, a))};
-}
-__device__ __forceinline__ DF df_add(DF a, DF b)
-{
-    float s, e, t, f;
-    two_sum(a.hi, b.hi, s, e);
-    two_sum(a.lo, b.lo, t, f);
-    DF r = quick_two_sum(s, __fadd_rn(e, t));
-    return quick_two_sum(r.hi, __fadd_rn(r.lo, f));
-}
-__device__ __forceinline__ DF df_add(DF a, float x)
-{
-    float s, e;
-    two_sum(a.hi, x, s, e);
-    return quick_two_sum(s, __fadd_rn(e, a.lo));
-}
-__device__ __forceinline__ DF df_mul(DF a, DF b)
-{
-    const float p = __fmul_rn(a.hi, b.hi);
-    const float e = __fmaf_rn(a.hi, b.hi, -p);
-    return quick_two_sum(p, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, e)));
-}
-__device__ __forceinline__ DF df_neg(DF a) { return {-a.hi, -a.lo}; }
-__device__ __forceinline__ double df_value(DF a) { return (double)a.hi + (double)a.lo; }
-__device__ __forceinline__ DF df_shfl_xor(DF a, int o)
-{
-    return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
-}
-
 // the six sums of a step: e2, e4, the potential (1 - phi^0 for the standard
 // model), det, |F|^2 and the sextic density e6 (zero without the sextic
 // term); plus max |F|^2
@@ -436,27 +259,6 @@ struct Acc {
     float s6, c6;     // e6 and its compensation (the sextic kernels)
     float f2, fmax2;
 };
-
-// the same for one quantity
-__device__ __forceinline__ void two_sum_acc1(float &s, float &c, float x)
-{
-    const float t = __fadd_rn(s, x);
-    const float bb = __fsub_rn(t, s);
-    c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(x, bb)));
-    s = t;
-}
-
-// s + x with the rounding error of the addition added to c (two quantities)
-__device__ __forceinline__ void two_sum_acc(float2 &s, float2 &c, float2 x)
-{
-    const float2 m1 = make_float2(-1.f, -1.f);
-    const float2 t = __fadd2_rn(s, x);
-    const float2 bb = __ffma2_rn(s, m1, t);                      // t - s
-    const float2 ea = __ffma2_rn(__ffma2_rn(bb, m1, t), m1, s);  // s - (t - bb)
-    const float2 eb = __ffma2_rn(bb, m1, x);                     // x - bb
-    c = __fadd2_rn(c, __fadd2_rn(ea, eb));
-    s = t;
-}
 
 // Fold a thread's running sums into its double-float sums, which live in
 // shared memory (acc: kSums arrays of stride nthreads, at this thread's slot).
@@ -519,16 +321,6 @@ __device__ __forceinline__ void block_reduce_df(DF (&v)[kSums], float amax, DF *
 #pragma unroll
         for (int q = 0; q < kSums; ++q) tot[q] = v[q];
         tmax = amax;
-    }
-}
-
-// Pairwise sum of x[0..K) into x[0] (K a power of two): a tree of depth log2 K
-template <int K> __device__ __forceinline__ void df_tree(DF (&x)[K])
-{
-#pragma unroll
-    for (int w = 1; w < K; w <<= 1) {
-#pragma unroll
-        for (int k = 0; k + w < K; k += 2 * w) x[k] = df_add(x[k], x[k + w]);
     }
 }
 
@@ -1528,39 +1320,6 @@ __global__ void __launch_bounds__(512, 2) k_fixup_batch(const InstDesc *__restri
     }
 }
 
-// ---------------------------------------------------- tensor maps
-static PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
-{
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    if (!fn) {
-        void *ptr = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &ptr, 12000,
-                                             cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(ptr);
-    }
-    return fn;
-}
-
-// 3D view (4 n2 floats, n1, n0) of a float4 site array; one box is a
-// box_z-float by box_y-row tile of a single x-plane.
-static bool make_plane_map(CUtensorMap *m, const void *base, const skyrme_lattice &lat,
-                           unsigned box_z, unsigned box_y)
-{
-    auto fn = encode_fn();
-    if (!fn) return false;
-    const cuuint64_t dims[3] = {(cuuint64_t)4 * lat.n[2], (cuuint64_t)lat.n[1], (cuuint64_t)lat.n[0]};
-    const cuuint64_t strides[2] = {(cuuint64_t)lat.n[2] * 16, (cuuint64_t)lat.n[1] * lat.n[2] * 16};
-    const cuuint32_t box[3] = {box_z, box_y, 1};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void *>(base), dims, strides,
-                    box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS;
-}
-
-
 // ------------------------------------------------------------------- host
 static int sm_count()
 {
@@ -1769,7 +1528,7 @@ static int grid_for(int tile, bool batched, long long units)
 bool f32_fast_path_available(const skyrme_lattice &lat)
 {
     // the streaming kernel needs the driver's tensor-map encoder
-    return lat.precision == 32 && encode_fn() != nullptr;
+    return lat.precision == 32 && tensor_map_encoder() != nullptr;
 }
 
 int f32_fast_blocks(const skyrme_lattice &lat)

@@ -1,7 +1,7 @@
 // flow_generic.cu -- tile-staged kernels of the arrested Newton flow in either
 // precision: the fused step (derivatives + Euler-Lagrange gradient + tangent
 // projection + velocity/field update + renormalisation + energy sums), the
-// speculative-arrest fix-up, the energy reduction and the per-site force dump.
+// speculative-arrest fix-up and the per-site force dump.
 //
 // One CTA owns a TX x TY x TZ block of interior sites and stages the field
 // with a 2-site halo in shared memory (Section 3: stencil radius 2).  The
@@ -217,7 +217,7 @@ __device__ __forceinline__ void normalise_store(vec4_t<T> *dst, const T t[4])
 // |F|^2 (max), e6}; the sextic sum is reduced only when EXT.
 template <typename T, bool EXT>
 __device__ __forceinline__ void reduce_and_finish(const FlowParams<T> &p, double (&acc)[7],
-                                                  bool energy_only, int pred)
+                                                  int pred)
 {
     __shared__ double red[8 * (GTHREADS / 32)];
     __shared__ int s_last;
@@ -234,8 +234,7 @@ __device__ __forceinline__ void reduce_and_finish(const FlowParams<T> &p, double
         rec[6] = 0.0;
         rec[7] = EXT ? tot6[NQ - 1] : 0.0;
         __threadfence();
-        unsigned int *ctr = energy_only ? &p.ctrl->edone : &p.ctrl->done;
-        const unsigned int t = atomicAdd(ctr, 1u);
+        const unsigned int t = atomicAdd(&p.ctrl->done, 1u);
         s_last = (t == (unsigned int)(nblocks - 1));
     }
     __syncthreads();
@@ -246,22 +245,7 @@ __device__ __forceinline__ void reduce_and_finish(const FlowParams<T> &p, double
     if (tid == 0) {
         const double nsites = (double)(p.n0 - 4) * (double)(p.n1 - 4) * (double)(p.n2 - 4);
         tot[6] = nsites;
-        if (energy_only) {
-            Ctrl *c = p.ctrl;
-            const double E2 = p.h3 * tot[0], E4 = p.h3 * tot[1], E0 = p.h3 * tot[2];
-            const double E6 = p.h3 * tot[7];
-            c->energy[0] = E2 + E4 + E0 + E6;
-            c->energy[1] = E2;
-            c->energy[2] = E4;
-            c->energy[3] = E0;
-            c->energy[4] = p.h3 * tot[3];
-            c->energy[5] = -E2 + E4 - 3.0 * E0 + 3.0 * E6;
-            c->e6_energy = E6;
-            c->energy[6] = sqrt(tot[5]);
-            c->energy[7] = sqrt(tot[4] / nsites);
-            if (!(isfinite(c->energy[0]) && isfinite(c->energy[4]))) c->status = DEV_NONFINITE;
-            c->edone = 0;
-        } else if (p.slab_rec) {
+        if (p.slab_rec) {
             // one x-slab of a larger lattice: the arrest decision needs every
             // slab's sums, so this step only leaves its record
 #pragma unroll
@@ -280,7 +264,7 @@ __device__ __forceinline__ void reduce_and_finish(const FlowParams<T> &p, double
 template <typename T, bool EXT>
 constexpr int kTileMinBlocks = sizeof(T) == 4 ? 3 : (EXT ? 1 : 2);
 
-// kind 0: fused step; kind 1: energy only; kind 2: per-site dump.
+// kind 0: fused step; kind 2: per-site dump.
 // EXT: the Section 7.8 extension terms are included.
 template <typename T, int KIND, bool EXT, int TZ>
 __global__ void __launch_bounds__(GTHREADS, kTileMinBlocks<T, EXT>) k_tile(FlowParams<T> p, vec4_t<T> *fout,
@@ -401,7 +385,7 @@ __global__ void __launch_bounds__(GTHREADS, kTileMinBlocks<T, EXT>) k_tile(FlowP
     }
     if (pending) fold();
     if (KIND == 2) return;
-    reduce_and_finish<T, EXT>(p, acc, KIND == 1, pred);
+    reduce_and_finish<T, EXT>(p, acc, pred);
 }
 
 // Pointwise correction of a mispredicted arrest decision: the step ran with
@@ -642,13 +626,6 @@ cudaError_t launch_step(const skyrme_lattice &lat, const FlowArgs &a, cudaStream
     if (lat.precision == 64)
         return launch_tile<double, 0>(lat, make_params<double>(a, a.step_parts), nullptr, nullptr, s);
     return launch_tile<float, 0>(lat, make_params<float>(a, a.step_parts), nullptr, nullptr, s);
-}
-
-cudaError_t launch_energy(const skyrme_lattice &lat, const FlowArgs &a, cudaStream_t s)
-{
-    if (lat.precision == 64)
-        return launch_tile<double, 1>(lat, make_params<double>(a, a.energy_parts), nullptr, nullptr, s);
-    return launch_tile<float, 1>(lat, make_params<float>(a, a.energy_parts), nullptr, nullptr, s);
 }
 
 cudaError_t launch_forces(const skyrme_lattice &lat, const FlowArgs &a, void *force, void *dens,

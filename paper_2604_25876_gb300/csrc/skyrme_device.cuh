@@ -64,7 +64,7 @@ struct Ctrl {
     int status;           // sticky status (0 or an error code)
     unsigned int done;    // arrival counter of the step launch
     unsigned int edone;   // arrival counter of the energy launch
-    double energy[8];     // E, E2, E4, E0, B, V, max|F|, rms|F| of skyrme_energy
+    double energy[8];     // E, E2, E4, E0, B, V of skyrme_energy (8 doubles of seed statistics)
     int hist;             // last 4 arrest decisions (bit 0 = latest)
     int pad_i;
     unsigned char pht[16];  // 2-bit saturating counters indexed by hist

@@ -1,0 +1,62 @@
+"""The passes over a whole field (energy, observables, render) at the sizes
+where their work splits have edges: lattices smaller than a tile or a chunk of
+planes, ragged sides, rows and planes one past a block, both z tiles."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_2604_25876_gb300 as sk
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+# smallest; one site past a 16- and a 32-wide z tile; odd rows; thin and long
+SIZES = [(5, 5, 5), (6, 5, 21), (9, 20, 37), (7, 21, 20), (70, 13, 6), (12, 40, 53), (8, 6, 300)]
+
+
+def field(n, h, seed=0, K=2):
+    rng = np.random.default_rng(seed)
+    pos = rng.uniform(-0.3, 0.3, size=(K, 3))
+    q = rng.normal(size=(K, 4))
+    q /= np.linalg.norm(q, axis=1, keepdims=True)
+    return oracle.seed_product(n, h, pos, q, 0.8, False)
+
+
+def on_gpu(phi, h, prec, **model):
+    lat = sk.Lattice(phi.shape[:3], h, 1.0, prec, **model)
+    st = sk.State(lat, DEV)
+    sk.load_field(lat, st, phi)
+    return lat, st, st.field().double().cpu().numpy()
+
+
+def determinant_scale(phi, h):
+    """Sum over the interior of the product of the determinant's row sizes /
+    2 pi^2: |phi| and, for each derivative, its norm and |phi| / h (a stencil's
+    rounding goes with the values it subtracts, not with their difference)."""
+    prod = np.linalg.norm(phi, axis=-1)[2:-2, 2:-2, 2:-2]
+    for ax in range(3):
+        s = [phi.take(np.arange(2 + o, phi.shape[ax] - 2 + o), axis=ax) for o in (-2, -1, 1, 2)]
+        d = (8 * (s[2] - s[1]) - (s[3] - s[0])) / (12 * h)
+        keep = tuple(slice(None) if a == ax else slice(2, -2) for a in range(3))
+        prod = prod * (np.linalg.norm(d, axis=-1)[keep] + 1.0 / h)
+    return prod.sum() / (2 * np.pi ** 2)
+
+
+# FP64: sums of at most 2e4 terms of one sign or of like size, each within a
+# few eps64 of the oracle's.  FP32: a density's rounding is about 20 eps32 of
+# its own size (stencil, products, minors), 1.2e-6, whatever the sums' signs.
+@pytest.mark.parametrize("n", SIZES)
+@pytest.mark.parametrize("prec,tol", [(64, 1e-12), (32, 2e-6)])
+@pytest.mark.parametrize("model", [{}, {"m_y": 0.5, "m_z": 0.3, "m_w": 1.0, "c6": 0.7}])
+def test_energy_matches_oracle_at_the_edges_of_the_work_split(n, prec, tol, model):
+    h = 0.25
+    lat, st, phi = on_gpu(field(n, h), h, prec, **model)
+    om = oracle.Model(1.0, *model.values()) if model else 1.0
+    eo, eg = oracle.energy(phi, h, om), sk.energy(lat, st)
+    for k in ("E", "E2", "E4", "E0"):
+        assert eg[k] == pytest.approx(eo[k], rel=tol, abs=tol * eo["E"]), k
+    # (where the lattice is one site wide B is nothing but rounding)
+    assert abs(eg["B"] - eo["B"]) <= tol * h ** 3 * determinant_scale(phi, h)
+    assert eg["virial"] == pytest.approx(eo["virial"], abs=5 * tol * eo["E"])
+    assert sk.energy(lat, st) == eg  # the same order every time
