@@ -60,3 +60,23 @@ def test_energy_matches_oracle_at_the_edges_of_the_work_split(n, prec, tol, mode
     assert abs(eg["B"] - eo["B"]) <= tol * h ** 3 * determinant_scale(phi, h)
     assert eg["virial"] == pytest.approx(eo["virial"], abs=5 * tol * eo["E"])
     assert sk.energy(lat, st) == eg  # the same order every time
+
+
+# (a lattice one site wide along an axis has no charge, so no observables)
+@pytest.mark.parametrize("n", [(6, 7, 21), (9, 20, 37), (7, 21, 20), (70, 13, 8), (12, 40, 53),
+                               (8, 9, 300)])
+@pytest.mark.parametrize("prec", [64, 32])
+def test_observables_match_oracle_at_the_edges_of_the_work_split(n, prec):
+    h = 0.25
+    lat, st, phi = on_gpu(field(n, h, 1), h, prec)
+    o, g = oracle.observables(phi, h, 1.0), sk.observables(lat, st)
+    # moments about X: scaled by the box and by |B|, which small boxes cut
+    box = h * max(n)
+    tol = (1e-10 if prec == 64 else 2e-6) * max(1.0, 1.0 / abs(o["B"]))
+    for k in ("B", "E"):
+        assert g[k] == pytest.approx(o[k], rel=tol), k
+    assert np.allclose(g["X"], o["X"], atol=tol * box, rtol=0)
+    for k in ("Q", "U", "V", "W"):
+        a, b = np.array(g[k]), np.array(o[k])
+        assert np.max(np.abs(a - b)) <= tol * max(1.0, np.max(np.abs(b))), k
+    assert g["D"] == pytest.approx(o["D"], abs=tol * o["E"] * max(1.0, np.max(np.abs(o["V"]))))
