@@ -790,9 +790,19 @@ skyrme_status skyrme_render(const skyrme_lattice *lat, skyrme_state *st,
     if (rc != SKYRME_OK) return rc;
     if (!params || !render_params_valid(*params) || !rgba || ((uintptr_t)rgba % 16))
         return SKYRME_EINVAL;
-    rc = skyrme_render_volume(lat, st, work, work_bytes, stream);
-    if (rc != SKYRME_OK) return rc;
-    return skyrme_render_rays(lat->n, work, params, rgba, stream);
+    if (!work || ((uintptr_t)work % 32)) return SKYRME_EINVAL;
+    if (work_bytes < skyrme_render_volume_bytes(lat)) return SKYRME_ENOMEM;
+    CKDEV(state_on_device(st));
+    {
+        const void *p[2] = {work, rgba};
+        CKDEV(on_current_device(p, 2));
+    }
+    const ScratchLayout L = scratch_layout(*lat);
+    FlowArgs a = make_args(*lat, *st, 0.0, MODE_ARRESTED);
+    CK(launch_render(*lat, a, *params, work, static_cast<char *>(st->scratch) + L.energy_off,
+                     L.total - L.energy_off, rgba, static_cast<cudaStream_t>(stream)),
+       "render");
+    return SKYRME_OK;
 }
 
 }  // extern "C"

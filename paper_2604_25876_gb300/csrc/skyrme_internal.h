@@ -93,10 +93,15 @@ size_t observables_parts_bytes();
 
 // Volume render of the baryon density (render.cu)
 bool render_params_valid(const skyrme_render_params &p);
+// (scratch: 256 bytes for the volume alone; a whole render uses as much of
+// scratch_bytes as its brick table needs)
 cudaError_t launch_render_volume(const skyrme_lattice &lat, const FlowArgs &a, void *vol,
-                                 void *bmax_scratch, cudaStream_t s);
+                                 void *scratch, cudaStream_t s);
 cudaError_t launch_render_rays(const int n[3], const void *vol, const skyrme_render_params &p,
                                float *rgba, cudaStream_t s);
+cudaError_t launch_render(const skyrme_lattice &lat, const FlowArgs &a,
+                          const skyrme_render_params &p, void *vol, void *scratch,
+                          size_t scratch_bytes, float *rgba, cudaStream_t s);
 
 // Seeds (init_fields.cu)
 cudaError_t launch_seed(const skyrme_lattice &lat, const skyrme_seed &seed, const FlowArgs &a,

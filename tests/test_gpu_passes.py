@@ -80,3 +80,61 @@ def test_observables_match_oracle_at_the_edges_of_the_work_split(n, prec):
         a, b = np.array(g[k]), np.array(o[k])
         assert np.max(np.abs(a - b)) <= tol * max(1.0, np.max(np.abs(b))), k
     assert g["D"] == pytest.approx(o["D"], abs=tol * o["E"] * max(1.0, np.max(np.abs(o["V"]))))
+
+
+def rotation(seed):
+    q = np.random.default_rng(seed).normal(size=4)
+    a, b, c, d = q / np.linalg.norm(q)
+    return np.array([[a * a + b * b - c * c - d * d, 2 * (b * c - a * d), 2 * (b * d + a * c)],
+                     [2 * (b * c + a * d), a * a - b * b + c * c - d * d, 2 * (c * d - a * b)],
+                     [2 * (b * d - a * c), 2 * (c * d + a * b), a * a - b * b - c * c + d * d]])
+
+
+@pytest.mark.parametrize("n", [(5, 6, 7), (33, 32, 35), (20, 90, 44), (66, 65, 64)])
+@pytest.mark.parametrize("view", [None, 1, 2])
+@pytest.mark.parametrize("levelset,scale,step", [(0.2, 4.0, 0.005), (0.6, 1.5, 0.011),
+                                                 (1e-3, 3.0, 0.02), (0.0, 1.0, 0.03),
+                                                 (0.3, -2.0, 0.02), (1.5, 4.0, 0.02)])
+def test_whole_render_equals_the_plain_march_bit_for_bit(n, view, levelset, scale, step):
+    """Samples passed over (by bricks, cells or the FP32 bound) change nothing:
+    the whole render, the rays on its volume and the oracle's plain march of
+    that volume give the same bits."""
+    h = 0.25
+    lat, st, _ = on_gpu(field(n, h, 4), h, 64)
+    p = dict(width=50, height=37, view=None if view is None else rotation(view),
+             levelset=levelset, transfer_scale=scale, step=step)
+    img = sk.render(lat, st, sk.render_params(**p))
+    vol = sk.render_volume(lat, st)
+    assert torch.equal(img, sk.render_rays(vol, sk.render_params(**p)))
+    ref = oracle.render_volume(vol.cpu().numpy(), **p).astype(np.float32)
+    assert np.array_equal(img.cpu().numpy(), ref)
+
+
+def test_rays_pass_over_no_sample_that_is_not_finite():
+    """Infinite and NaN densities count as the plain march counts them."""
+    rng = np.random.default_rng(2)
+    vol = rng.uniform(0.0, 0.15, size=(24, 22, 26, 4))
+    vol[7, 8, 9, 0], vol[15, 11, 12, 0], vol[12, 5, 20, 0], vol[18, 18, 3, 0] = np.nan, np.inf, -np.inf, 0.9
+    p = dict(width=61, height=47, levelset=0.2, step=0.01)
+    img = sk.render_rays(torch.from_numpy(vol).to(DEV), sk.render_params(**p)).cpu().numpy()
+    ref = oracle.render_volume(vol, **p).astype(np.float32)
+    assert np.array_equal(img, ref, equal_nan=True)
+
+
+def test_volume_quotients_are_correctly_rounded_over_the_range():
+    """pion / |pion| of tiny, huge-ratio and denormal pions: IEEE quotients."""
+    rng = np.random.default_rng(8)
+    n = (12, 13, 14)
+    phi = np.zeros(n + (4,))
+    phi[..., 0] = 1.0
+    mag = 10.0 ** rng.uniform(-300, 0, size=n + (3,))
+    phi[..., 1:] = mag * rng.choice([-1.0, 1.0, 0.0], size=n + (3,))
+    lat, st, got_phi = on_gpu(phi, 0.25, 64)
+    vol = sk.render_volume(lat, st).cpu().numpy()
+    ref = oracle.render_volume_from_field(got_phi, 0.25)
+    assert np.array_equal(vol[..., 1:], ref[..., 1:])
+    # an FP32 field with denormals (the widening's rare branch)
+    lat, st, got_phi = on_gpu((10.0 ** rng.uniform(-44, 0, size=n + (4,))).astype(np.float32), 0.25, 32)
+    vol = sk.render_volume(lat, st).cpu().numpy()
+    ref = oracle.render_volume_from_field(got_phi, 0.25)
+    assert np.array_equal(vol[..., 1:], ref[..., 1:])
