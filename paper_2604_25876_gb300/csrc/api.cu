@@ -266,7 +266,8 @@ skyrme_status skyrme_init_field(const skyrme_lattice *lat, const skyrme_seed *se
     FlowArgs a = make_args(*lat, *st, 0.0, MODE_ARRESTED);
     CK(launch_reset_ctrl(a.ctrl, s), "reset control block");
     CK(launch_seed(*lat, *seed, a, s), "seed kernels");
-    CK(launch_load_finish(*lat, a, s), "finish field");
+    // (the product seed writes the whole state itself)
+    if (seed->kind != SKYRME_SEED_PRODUCT) CK(launch_load_finish(*lat, a, s), "finish field");
     return SKYRME_OK;
 }
 

@@ -138,3 +138,29 @@ def test_volume_quotients_are_correctly_rounded_over_the_range():
     vol = sk.render_volume(lat, st).cpu().numpy()
     ref = oracle.render_volume_from_field(got_phi, 0.25)
     assert np.array_equal(vol[..., 1:], ref[..., 1:])
+
+
+# below and above the size from which the profile is tabulated; a constituent
+# on a lattice site; radii past the table's last interval (rho = 57); a scale
+# that is no power of two
+@pytest.mark.parametrize("n,h,K,scale", [((9, 12, 33), 0.25, 3, 1.0), ((110, 100, 96), 0.3, 1, 0.5),
+                                         ((101, 99, 103), 0.2, 2, 1.7)])
+@pytest.mark.parametrize("prec", [64, 32])
+@pytest.mark.parametrize("sym", [True, False])
+def test_product_seed_matches_oracle(n, h, K, scale, prec, sym):
+    rng = np.random.default_rng(K)
+    pos = rng.uniform(-1.0, 1.0, size=(K, 3))
+    pos[0] = [(n[a] // 2 - 0.5 * (n[a] - 1)) * h for a in range(3)]  # r = 0 at a site
+    q = rng.normal(size=(K, 4))
+    q /= np.linalg.norm(q, axis=1, keepdims=True)
+    lat = sk.Lattice(n, h, 1.0, prec)
+    st = sk.State(lat, DEV)
+    st.vel.fill_(3.0)
+    sk.init_field(lat, sk.Seed.product(pos, q, scale, sym), st)
+    ref = oracle.seed_product(n, h, pos, q, scale, sym)
+    # 64 bits: a few eps per constituent, times the radius in the exponent
+    # (symmetrised: over the norm of the sum, above 1e-3 here); 32: rounding
+    got = st.phi[0].double().cpu().numpy()
+    assert np.max(np.abs(got - ref)) <= (1e-12 if prec == 64 else 1.2e-7)
+    assert torch.equal(st.phi[0], st.phi[1]) and not st.vel.any().item()
+    assert sk.read_report(lat, st)["steps"] == 0
