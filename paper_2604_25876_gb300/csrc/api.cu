@@ -301,8 +301,10 @@ static skyrme_status launch_iterations(const skyrme_lattice &lat, const FlowArgs
     }
     for (int k = 0; k < nsteps; ++k) {
         CK(launch_step(lat, a, s), "step kernel");
-        // an x-slab's fix-up follows the decision over all slabs
-        if (a.mode == SKYRME_ARRESTED && !a.slab_rec) CK(launch_fixup(lat, a, s), "fix-up kernel");
+        // the FP64 step corrects its own sites; an x-slab's fix-up follows the
+        // decision over all slabs
+        if (lat.precision == 32 && a.mode == SKYRME_ARRESTED && !a.slab_rec)
+            CK(launch_fixup(lat, a, s), "fix-up kernel");
     }
     return SKYRME_OK;
 }

@@ -693,10 +693,6 @@ __device__ __forceinline__ void write_record(const InstDesc &D, int slot, const 
     recp[3] = make_float4(tot[5].hi, tot[5].lo, 0.f, 0.f);
 }
 
-__device__ __forceinline__ void st_release_s64(long long *p, long long v)
-{
-    asm volatile("st.release.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
 // Arrival at a lattice's counter: releases this thread's earlier stores (the
 // CTA record) and acquires every earlier arrival's
 __device__ __forceinline__ unsigned atom_add_acq_rel(unsigned *p, unsigned v)
@@ -871,13 +867,6 @@ __device__ __forceinline__ void finish_lattice(const InstDesc &D, Ctrl *c, int c
         c->e6_last = df_value(E6);
         if (!(isfinite(Ed) && isfinite(B.hi) && isfinite(t[4].hi))) c->status = DEV_NONFINITE;
     }
-}
-
-__device__ __forceinline__ long long ld_acquire_s64(const long long *p)
-{
-    long long v;
-    asm volatile("ld.acquire.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
 }
 
 // The step's own correction of a mispredicted arrest decision, at the sites

@@ -426,7 +426,13 @@ template <typename T> __global__ void __launch_bounds__(512, 2) k_fixup(FlowPara
 #pragma unroll
             for (int k = 0; k < kFixUnroll; ++k) {
                 const int z = z0 + 32 * k + lane;
-                if (z < iz) {
+                if (z >= iz) continue;
+                if constexpr (sizeof(T) == 8) {
+                    vec4_t<T> v, f;
+                    arrest_fix_site(vn[k], vo[k], fo[k], sgn, p.dt, v, f);
+                    store4<T>(vnew + base + z, v);
+                    store4<T>(pnew + base + z, f);
+                } else {
                     const T v0 = vn[k].x + sgn * vo[k].x, v1 = vn[k].y + sgn * vo[k].y;
                     const T v2 = vn[k].z + sgn * vo[k].z, v3 = vn[k].w + sgn * vo[k].w;
                     const T t0 = fo[k].x + p.dt * v0, t1 = fo[k].y + p.dt * v1;
@@ -623,8 +629,7 @@ static cudaError_t launch_tile(const skyrme_lattice &lat, const FlowParams<T> &p
 
 cudaError_t launch_step(const skyrme_lattice &lat, const FlowArgs &a, cudaStream_t s)
 {
-    if (lat.precision == 64)
-        return launch_tile<double, 0>(lat, make_params<double>(a, a.step_parts), nullptr, nullptr, s);
+    if (lat.precision == 64) return launch_step_f64(lat, a, s);
     return launch_tile<float, 0>(lat, make_params<float>(a, a.step_parts), nullptr, nullptr, s);
 }
 

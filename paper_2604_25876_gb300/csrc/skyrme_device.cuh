@@ -396,39 +396,100 @@ __device__ __forceinline__ void reduce_partials(const double *parts, int nparts,
     }
 }
 
-// End-of-step bookkeeping, run by thread 0 of the last CTA to arrive (or,
-// for a lattice split into x-slabs, by the one-thread kernel that combines the
-// slabs' records).
-// tot = {sum e2, sum e4, sum e0, sum b, sum |F|^2, max |F|^2, n_sites, sum e6}.
-__device__ __forceinline__ void finish_step(Ctrl *c, const double (&tot)[kPartialDoubles],
-                                            double h3, int mode, int pred)
+// Publication of a step: a release store, and the acquire load of those who wait
+__device__ __forceinline__ void st_release_s64(long long *p, long long v)
 {
-    const double E2 = h3 * tot[0], E4 = h3 * tot[1], E0 = h3 * tot[2], E6 = h3 * tot[7];
-    const double E = E2 + E4 + E0 + E6;
-    const double B = h3 * tot[3];
-    const double delta = sqrt(tot[5]);
-    const double rms = tot[6] > 0.0 ? sqrt(tot[4] / tot[6]) : 0.0;
+    asm volatile("st.release.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ long long ld_acquire_s64(const long long *p)
+{
+    long long v;
+    asm volatile("ld.acquire.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// One FP64 site of the correction of a mispredicted arrest decision:
+// v = v_new + sgn v_old, phi = normalise(phi_old + dt v), every operation
+// rounded explicitly, so that every path that corrects a site (the step's own
+// correction, an x-slab's fix-up) gives the same bits.
+__device__ __forceinline__ void arrest_fix_site(const dvec4 &vn, const dvec4 &vo, const dvec4 &fo, double sgn,
+                                                double dt, dvec4 &v, dvec4 &f)
+{
+    v = dvec4{__fma_rn(sgn, vo.x, vn.x), __fma_rn(sgn, vo.y, vn.y), __fma_rn(sgn, vo.z, vn.z),
+              __fma_rn(sgn, vo.w, vn.w)};
+    const dvec4 t = {__fma_rn(dt, v.x, fo.x), __fma_rn(dt, v.y, fo.y), __fma_rn(dt, v.z, fo.z),
+                     __fma_rn(dt, v.w, fo.w)};
+    const double r = rsqrt(__fma_rn(t.w, t.w, __fma_rn(t.z, t.z, __fma_rn(t.y, t.y, __dmul_rn(t.x, t.x)))));
+    f = dvec4{__dmul_rn(t.x, r), __dmul_rn(t.y, r), __dmul_rn(t.z, r), __dmul_rn(t.w, r)};
+}
+
+// End-of-step bookkeeping, run by the last CTA to arrive (or, for a lattice
+// split into x-slabs, by the one-thread kernel that combines the slabs'
+// records).  tot = {sum e2, sum e4, sum e0, sum b, sum |F|^2, max |F|^2,
+// n_sites, sum e6}.
+
+// The control fields that the decision needs (loads independent of the sums)
+struct StepControl {
+    double E_prev;
+    long long steps, arrests, fixups;
+    int hist, cur;
+    uint4 pht;
+};
+__device__ __forceinline__ StepControl load_control(const Ctrl *c)
+{
+    StepControl s;
+    s.E_prev = __ldcg(&c->E_prev);
+    s.steps = __ldcg(&c->steps);
+    s.arrests = __ldcg(&c->arrests);
+    s.fixups = __ldcg(&c->fixups);
+    s.hist = __ldcg(&c->hist);
+    s.cur = __ldcg(&c->cur);
+    s.pht = __ldcg(reinterpret_cast<const uint4 *>(c->pht));
+    return s;
+}
+__device__ __forceinline__ double step_energy(const double (&tot)[kPartialDoubles], double h3)
+{
+    return h3 * tot[0] + h3 * tot[1] + h3 * tot[2] + h3 * tot[7];
+}
+// The arrest decision, the predictor and the published step count.
+__device__ __forceinline__ void decide_step(Ctrl *c, const StepControl &s,
+                                            const double (&tot)[kPartialDoubles], double h3, int mode,
+                                            int pred)
+{
+    const double E = step_energy(tot, h3);
     int actual = 0;
-    if (mode == MODE_ARRESTED) actual = (E > c->E_prev) ? 1 : 0;
+    if (mode == MODE_ARRESTED) actual = (E > s.E_prev) ? 1 : 0;
     const int fix = (actual == pred) ? 0 : (actual ? -1 : +1);
-    c->fix = fix;
     // two-level adaptive prediction of the next decision: the last four
     // decisions select a 2-bit saturating counter (learns runs and the
-    // alternating arrest pattern of a nearly converged flow)
-    {
-        const int h = c->hist & 15;
-        int ctr = c->pht[h];
-        ctr = actual ? (ctr < 3 ? ctr + 1 : 3) : (ctr > 0 ? ctr - 1 : 0);
-        c->pht[h] = (unsigned char)ctr;
-        const int hn = ((h << 1) | actual) & 15;
-        c->hist = hn;
-        c->pred = c->pht[hn] >= 2 ? 1 : 0;
-    }
-    c->arrests += actual;
-    c->fixups += (fix != 0);
+    // alternating arrest pattern of a nearly converged flow); counter i of the
+    // 16 is byte i of pht (read by shifts, no local copy)
+    auto counter = [&](int i) {
+        const unsigned w = i < 8 ? (i < 4 ? s.pht.x : s.pht.y) : (i < 12 ? s.pht.z : s.pht.w);
+        return (int)((w >> (8 * (i & 3))) & 0xffu);
+    };
+    const int h = s.hist & 15;
+    int ctr = counter(h);
+    ctr = actual ? (ctr < 3 ? ctr + 1 : 3) : (ctr > 0 ? ctr - 1 : 0);
+    const int hn = ((h << 1) | actual) & 15;
+    c->fix = fix;
+    c->pht[h] = (unsigned char)ctr;
+    c->hist = hn;
+    c->pred = (h == hn ? ctr : counter(hn)) >= 2 ? 1 : 0;
+    c->arrests = s.arrests + actual;
+    c->fixups = s.fixups + (fix != 0);
     c->E_prev = E;
-    c->steps += 1;
-    c->cur ^= 1;
+    c->cur = s.cur ^ 1;
+    c->done = 0;
+    // the step count goes last, released: CTAs that correct their own sites
+    // wait for it, and then see every field above
+    st_release_s64(&c->steps, s.steps + 1);
+}
+// The reported values, which no CTA waits for.
+__device__ __forceinline__ void report_step(Ctrl *c, const double (&tot)[kPartialDoubles], double h3)
+{
+    const double E2 = h3 * tot[0], E4 = h3 * tot[1], E0 = h3 * tot[2], E6 = h3 * tot[7];
+    const double E = step_energy(tot, h3), B = h3 * tot[3];
     c->last[0] = E;
     c->last[1] = E2;
     c->last[2] = E4;
@@ -436,10 +497,15 @@ __device__ __forceinline__ void finish_step(Ctrl *c, const double (&tot)[kPartia
     c->last[4] = B;
     c->last[5] = -E2 + E4 - 3.0 * E0 + 3.0 * E6;
     c->e6_last = E6;
-    c->last[6] = delta;
-    c->last[7] = rms;
+    c->last[6] = sqrt(tot[5]);
+    c->last[7] = tot[6] > 0.0 ? sqrt(tot[4] / tot[6]) : 0.0;
     if (!(isfinite(E) && isfinite(B) && isfinite(tot[4]))) c->status = DEV_NONFINITE;
-    c->done = 0;
+}
+__device__ __forceinline__ void finish_step(Ctrl *c, const double (&tot)[kPartialDoubles], double h3,
+                                            int mode, int pred)
+{
+    decide_step(c, load_control(c), tot, h3, mode, pred);
+    report_step(c, tot, h3);
 }
 
 }  // namespace skyrme

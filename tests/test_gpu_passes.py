@@ -164,3 +164,28 @@ def test_product_seed_matches_oracle(n, h, K, scale, prec, sym):
     assert np.max(np.abs(got - ref)) <= (1e-12 if prec == 64 else 1.2e-7)
     assert torch.equal(st.phi[0], st.phi[1]) and not st.vel.any().item()
     assert sk.read_report(lat, st)["steps"] == 0
+
+
+# the FP64 step's columns (2 x 16 or 4 x 8), runs and shares: lattices of fewer
+# units than warps, runs that cross columns, both column shapes, long runs
+@pytest.mark.parametrize("n", SIZES + [(33, 48, 48), (200, 14, 18)])
+@pytest.mark.parametrize("mode", [sk.ARRESTED, sk.NEWTON, sk.GRADIENT])
+@pytest.mark.parametrize("model", [{}, {"m_y": 0.5, "m_z": 0.3, "m_w": 1.0, "c6": 0.02}])
+def test_fp64_steps_match_oracle_at_the_edges_of_the_work_split(n, mode, model):
+    h, dt, steps = 0.25, 0.004, 6
+    lat, st, phi = on_gpu(field(n, h, 2), h, 64, **model)
+    om = oracle.Model(1.0, *model.values()) if model else 1.0
+    ost = oracle.new_state(phi)
+    reps = oracle.flow(ost, h, om, dt, steps, mode=mode, reports=True)
+    rep = sk.flow_step(lat, dt, steps, mode, st)
+    # a few hundred roundings of the forces (up to 1e3 here) times dt, six steps
+    assert np.max(np.abs(st.field().cpu().numpy() - ost.phi)) <= 1e-11
+    if mode != sk.GRADIENT:
+        scale = max(1.0, np.max(np.abs(ost.v)))
+        assert np.max(np.abs(st.velocity().cpu().numpy() - ost.v)) <= 1e-11 * scale
+    # (1 - phi^0 is rounded to eps of 1, not of itself: a converged field's
+    # energy is a sum of such roundings)
+    eps_sum = 1e-15 * h ** 3 * np.prod([v - 4 for v in n])
+    for k in ("E", "E2", "E4", "E0"):
+        assert rep[k] == pytest.approx(reps[-1][k], rel=1e-11, abs=1e-11 * reps[-1]["E"] + eps_sum), k
+    assert rep["steps"] == steps and rep["status"] == 0
