@@ -144,6 +144,14 @@ skyrme_status skyrme_init_field(const skyrme_lattice *lat, const skyrme_seed *se
  * copied to phi[1], its outer layers are set to the vacuum, velocities are
  * zeroed and the control block reset, as after skyrme_init_field. */
 skyrme_status skyrme_load_field(const skyrme_lattice *lat, skyrme_state *st, void *stream);
+/* skyrme_load_field_from: the same from a field `src` in the caller's memory
+ * (device, or host memory the device can address; layout, precision and
+ * alignment of phi), which is read once and must stay valid until the call's
+ * work on `stream` is done: it saves the caller's copy into phi[0].
+ * SKYRME_EINVAL when src is null or misaligned or overlaps the state's
+ * buffers. */
+skyrme_status skyrme_load_field_from(const skyrme_lattice *lat, skyrme_state *st, const void *src,
+                                     void *stream);
 
 /* ---- the flow (Section 3) ----
  * nsteps iterations of `mode` with time step dt > 0.  One iteration computes

@@ -84,6 +84,8 @@ _SIGNATURES = {
     "skyrme_init_field": (ctypes.c_int, [ctypes.POINTER(c_lattice), ctypes.POINTER(c_seed),
                                          ctypes.POINTER(c_state), _P]),
     "skyrme_load_field": (ctypes.c_int, [ctypes.POINTER(c_lattice), ctypes.POINTER(c_state), _P]),
+    "skyrme_load_field_from": (ctypes.c_int, [ctypes.POINTER(c_lattice), ctypes.POINTER(c_state), _P,
+                                              _P]),
     "skyrme_flow_step": (ctypes.c_int, [ctypes.POINTER(c_lattice), ctypes.c_double, ctypes.c_int,
                                         ctypes.c_int, ctypes.POINTER(c_state),
                                         ctypes.POINTER(c_report), _P]),
@@ -355,13 +357,38 @@ def init_field(lat: Lattice, seed: Seed, st: State, stream=None):
     del keep
 
 
+def _loadable(lat: Lattice, st: State, t) -> bool:
+    """Whether the load kernel can read the tensor where it is: a plain
+    contiguous tensor of the state's device, precision and shape, aligned to a
+    site and apart from the state's buffers."""
+    torch = _torch()
+    if type(t) is not torch.Tensor or not t.is_cuda or t.device != st.phi.device or \
+            t.dtype != lat.dtype or t.shape != st.phi.shape[1:] or not t.is_contiguous() or \
+            t.requires_grad or t.is_neg() or t.numel() == 0:
+        return False
+    site, a = 4 * t.element_size(), t.data_ptr()
+    b = a + t.numel() * t.element_size()
+    for buf in (st.phi, st.vel):
+        lo = buf.data_ptr()
+        if a < lo + buf.numel() * buf.element_size() and lo < b:
+            return False
+    return a % site == 0
+
+
 def load_field(lat: Lattice, st: State, phi, stream=None):
     """Start a flow from a given field (any device/host tensor or array of
     shape (Nx, Ny, Nz, 4)); its outer layers are replaced by the vacuum."""
     torch = _torch()
     t = torch.as_tensor(np.asarray(phi) if not isinstance(phi, torch.Tensor) else phi)
-    st.phi[0].copy_(t.to(device=st.device, dtype=lat.dtype))
     cl, cs = lat.c(), st.c()
+    if stream is None and _loadable(lat, st, t):
+        # read by the load kernel itself, on the current stream as the copy is
+        _check(_on(st.device).skyrme_load_field_from(ctypes.byref(cl), ctypes.byref(cs),
+                                                     ctypes.c_void_p(t.data_ptr()),
+                                                     _stream_ptr(None, st.device)),
+               "skyrme_load_field_from")
+        return
+    st.phi[0].copy_(t.to(device=st.device, dtype=lat.dtype))
     _check(_on(st.device).skyrme_load_field(ctypes.byref(cl), ctypes.byref(cs),
                                     _stream_ptr(stream, st.device)), "skyrme_load_field")
 

@@ -283,6 +283,27 @@ skyrme_status skyrme_load_field(const skyrme_lattice *lat, skyrme_state *st, voi
     return SKYRME_OK;
 }
 
+skyrme_status skyrme_load_field_from(const skyrme_lattice *lat, skyrme_state *st, const void *src,
+                                     void *stream)
+{
+    skyrme_status rc = check_state(lat, st);
+    if (rc != SKYRME_OK) return rc;
+    const size_t align = site_bytes(*lat);
+    if (!src || ((uintptr_t)src % align)) return SKYRME_EINVAL;
+    const uintptr_t bytes = (uintptr_t)lat->n[0] * lat->n[1] * lat->n[2] * align;
+    for (int i = 0; i < 4; ++i) {
+        const uintptr_t b = (uintptr_t)(i < 2 ? st->phi[i] : st->vel[i - 2]), f = (uintptr_t)src;
+        if (f < b + bytes && b < f + bytes) return SKYRME_EINVAL;
+    }
+    CKDEV(state_on_device(st));
+    CKDEV(on_current_device(&src, 1));
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    FlowArgs a = make_args(*lat, *st, 0.0, MODE_ARRESTED);
+    CK(launch_reset_ctrl(a.ctrl, s), "reset control block");
+    CK(launch_load_finish(*lat, a, s, src), "load field");
+    return SKYRME_OK;
+}
+
 // FP32 flows run on the streaming kernel (the standard model, the Section 7.8
 // potentials and the sextic term)
 static bool fp32_streaming(const skyrme_lattice &lat)

@@ -446,25 +446,44 @@ template <typename T> __global__ void __launch_bounds__(512, 2) k_fixup(FlowPara
     }
 }
 
-// phi[1] <- phi[0] (read from src instead when it is given: a caller's field
-// in pinned host memory, read over the host link); outer layers <- vacuum in
-// both; velocities <- 0.
-template <typename T> __global__ void k_load_finish(FlowParams<T> p, const vec4_t<T> *src)
+// The state of a field just loaded: phi[1] <- phi[0], the outer layers of both
+// the vacuum, velocities 0.  With a source (a caller's field on the device, or
+// in pinned host memory and then read over the host link) phi[0] <- src too;
+// without one the interior of phi[0] is not written again.
+// Bound by DRAM: one buffer read and three (with a source four) written.
+// 512^3 FP32, after a copy of the caller's field into phi[0] and with phi[0]
+// rewritten, before: MEASURED
+template <typename T, bool SRC>
+__global__ void __launch_bounds__(256) k_load_field(FlowParams<T> p, const vec4_t<T> *__restrict__ src)
 {
-    const vec4_t<T> *in = src ? src : p.phi[0];
-    const size_t total = (size_t)p.n0 * p.n1 * p.n2;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const int z = (int)(i % p.n2);
-        const int y = (int)((i / p.n2) % p.n1);
-        const int x = (int)(i / ((size_t)p.n2 * p.n1));
-        const bool inner = x >= 2 && x <= p.n0 - 3 && y >= 2 && y <= p.n1 - 3 && z >= 2 &&
-                           z <= p.n2 - 3;
-        vec4_t<T> f = inner ? load4<T>(in + i) : make4<T>(T(1), T(0), T(0), T(0));
-        store4<T>(p.phi[0] + i, f);
-        store4<T>(p.phi[1] + i, f);
-        store4<T>(p.vel[0] + i, make4<T>(T(0), T(0), T(0), T(0)));
-        store4<T>(p.vel[1] + i, make4<T>(T(0), T(0), T(0), T(0)));
+    constexpr int kPer = 4;  // sites per thread and pass
+    const vec4_t<T> vac = make4<T>(T(1), T(0), T(0), T(0)), zero = make4<T>(T(0), T(0), T(0), T(0));
+    const unsigned plane = (unsigned)p.n1 * p.n2, blocks = (plane + 256 * kPer - 1) / (256 * kPer);
+    const unsigned items = blocks * p.n0;
+    const vec4_t<T> *in = SRC ? src : p.phi[0];
+    for (unsigned it = blockIdx.x; it < items; it += gridDim.x) {
+        const unsigned x = it / blocks, i0 = (it - x * blocks) * 256 * kPer + threadIdx.x;
+        const bool xin = (int)x >= 2 && (int)x <= p.n0 - 3;
+        const size_t s0 = (size_t)x * plane;
+        vec4_t<T> f[kPer];
+        bool inner[kPer];
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            const unsigned i = i0 + 256 * k;
+            const int y = (int)(i / (unsigned)p.n2), z = (int)(i - (unsigned)y * p.n2);
+            inner[k] = xin && i < plane && y >= 2 && y <= p.n1 - 3 && z >= 2 && z <= p.n2 - 3;
+            f[k] = vac;
+            if (inner[k]) f[k] = load4<T>(in + s0 + i);
+        }
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            const unsigned i = i0 + 256 * k;
+            if (i >= plane) continue;
+            if (SRC || !inner[k]) store4<T>(p.phi[0] + s0 + i, f[k]);
+            store4<T>(p.phi[1] + s0 + i, f[k]);
+            store4<T>(p.vel[0] + s0 + i, zero);
+            store4<T>(p.vel[1] + s0 + i, zero);
+        }
     }
 }
 
@@ -643,14 +662,6 @@ cudaError_t launch_forces(const skyrme_lattice &lat, const FlowArgs &a, void *fo
                                  static_cast<float4 *>(force), static_cast<float4 *>(dens), s);
 }
 
-static int pointwise_blocks(size_t total)
-{
-    size_t b = (total + 255) / 256;
-    if (b > 152 * 16) b = 152 * 16;
-    if (b < 1) b = 1;
-    return (int)b;
-}
-
 cudaError_t launch_fixup(const skyrme_lattice &lat, const FlowArgs &a, cudaStream_t s)
 {
     // mostly an early exit: one wave of 512-thread blocks, 16 rows each at most per pass
@@ -663,17 +674,22 @@ cudaError_t launch_fixup(const skyrme_lattice &lat, const FlowArgs &a, cudaStrea
     return cudaGetLastError();
 }
 
+template <typename T>
+static cudaError_t launch_load(const FlowArgs &a, const void *src, cudaStream_t s)
+{
+    const FlowParams<T> p = make_params<T>(a, a.step_parts);
+    const long long items = (long long)a.n[0] * (((long long)a.n[1] * a.n[2] + 1023) / 1024);
+    const int grid = (int)std::min<long long>(items, 152 * 8);
+    const vec4_t<T> *f = static_cast<const vec4_t<T> *>(src);
+    if (src) k_load_field<T, true><<<grid, 256, 0, s>>>(p, f);
+    else k_load_field<T, false><<<grid, 256, 0, s>>>(p, nullptr);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_load_finish(const skyrme_lattice &lat, const FlowArgs &a, cudaStream_t s,
                                const void *src)
 {
-    const size_t total = (size_t)lat.n[0] * lat.n[1] * lat.n[2];
-    if (lat.precision == 64)
-        k_load_finish<double><<<pointwise_blocks(total), 256, 0, s>>>(
-            make_params<double>(a, a.step_parts), static_cast<const vec4_t<double> *>(src));
-    else
-        k_load_finish<float><<<pointwise_blocks(total), 256, 0, s>>>(
-            make_params<float>(a, a.step_parts), static_cast<const vec4_t<float> *>(src));
-    return cudaGetLastError();
+    return lat.precision == 64 ? launch_load<double>(a, src, s) : launch_load<float>(a, src, s);
 }
 
 cudaError_t launch_reset_ctrl(void *ctrl, cudaStream_t s)

@@ -189,3 +189,48 @@ def test_fp64_steps_match_oracle_at_the_edges_of_the_work_split(n, mode, model):
     for k in ("E", "E2", "E4", "E0"):
         assert rep[k] == pytest.approx(reps[-1][k], rel=1e-11, abs=1e-11 * reps[-1]["E"] + eps_sum), k
     assert rep["steps"] == steps and rep["status"] == 0
+
+
+@pytest.mark.parametrize("n", SIZES + [(6, 40, 52)])
+@pytest.mark.parametrize("prec", [64, 32])
+def test_load_field_gives_the_same_state_from_every_source(n, prec):
+    """The direct read, the copy (host, other layout, other type, an offset
+    that breaks the alignment, the state's own buffers) and the two outer
+    layers, over the edges of the load kernel's blocks."""
+    lat = sk.Lattice(n, 0.25, 1.0, prec)
+    phi = field(n, 0.25, 3)
+    ref = oracle.apply_vacuum_boundary(phi.copy())
+    ref = torch.from_numpy(ref if prec == 64 else ref.astype(np.float32)).to(DEV)
+    t = torch.from_numpy(phi).to(DEV, lat.dtype)
+    odd = torch.empty(t.numel() + 1, dtype=lat.dtype, device=DEV)[1:].view(t.shape).copy_(t)
+    sources = [t, phi, t.cpu(), t.transpose(0, 1).contiguous().transpose(0, 1), t.double(), odd,
+               t.clone().requires_grad_(), -(-t)]
+    for src in sources + ["own 0", "own 1"]:
+        st = sk.State(lat, DEV)
+        st.phi.fill_(0.5)
+        st.vel.fill_(0.5)
+        st.scratch.fill_(7)
+        if isinstance(src, str):
+            src, _ = st.phi[int(src[-1])], st.phi[int(src[-1])].copy_(t)
+        with torch.no_grad():
+            sk.load_field(lat, st, src)
+        assert torch.equal(st.phi[0], ref) and torch.equal(st.phi[1], ref)
+        assert not st.vel.any().item()
+        rep = sk.read_report(lat, st)
+        assert rep["steps"] == 0 and rep["cur"] == 0 and rep["status"] == 0
+    with pytest.raises(RuntimeError):  # shapes that do not broadcast stay refused
+        sk.load_field(lat, sk.State(lat, DEV), t[1:])
+
+
+def test_load_field_from_rejects_null_misaligned_and_overlapping_sources():
+    import ctypes
+    lat = sk.Lattice((6, 7, 8), 0.25, 1.0, 32)
+    st = sk.State(lat, DEV)
+    cl, cs = lat.c(), st.c()
+    f = torch.zeros(6 * 7 * 8 * 4 + 4, device=DEV)
+    call = lambda p: sk.load().skyrme_load_field_from(ctypes.byref(cl), ctypes.byref(cs),  # noqa: E731
+                                                      ctypes.c_void_p(p), None)
+    assert call(None) == 1 and call(f.data_ptr() + 4) == 1
+    assert call(st.phi[0].data_ptr() + 16) == 1 and call(st.vel[1].data_ptr()) == 1
+    assert call(f.data_ptr() + 16) == 0
+    torch.cuda.synchronize()
