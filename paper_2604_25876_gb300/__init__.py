@@ -60,8 +60,11 @@ class c_seed(ctypes.Structure):
                 ("sigma", ctypes.c_double), ("seed", ctypes.c_uint64)]
 
 
+_VoidP2 = ctypes.c_void_p * 2
+
+
 class c_state(ctypes.Structure):
-    _fields_ = [("phi", ctypes.c_void_p * 2), ("vel", ctypes.c_void_p * 2),
+    _fields_ = [("phi", _VoidP2), ("vel", _VoidP2),
                 ("scratch", ctypes.c_void_p), ("scratch_bytes", ctypes.c_size_t)]
 
 
@@ -187,9 +190,15 @@ def _check(rc: int, where: str):
         raise SkyrmeError(rc, where, detail)
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 class _On:
@@ -210,14 +219,25 @@ class _On:
         return call
 
 
-def _on(device) -> _On:
+def _on(device):
+    """The library's functions for buffers on ``device``: the library itself
+    when that is the current device (a device context costs 3 us a call)."""
+    i = device.index
+    if i is None or i == _torch().cuda.current_device():
+        return _lib if _lib is not None else load()
     return _On(device)
 
 
 def _stream_ptr(stream=None, device=None):
     torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream(device)
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return ctypes.c_void_p(stream.cuda_stream)
+    i = device.index if device is not None else None
+    if i is None:
+        i = torch.cuda.current_device()
+    # the handle alone: a Stream object costs 3.5 us a call
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return ctypes.c_void_p(raw(i) if raw is not None else torch.cuda.current_stream(i).cuda_stream)
 
 
 # --------------------------------------------------------------- lattice
@@ -329,10 +349,12 @@ class State:
         self.scratch = torch.zeros(lat.scratch_bytes(), dtype=torch.uint8, device=self.device)
 
     def c(self) -> c_state:
-        return c_state((ctypes.c_void_p * 2)(self.phi[0].data_ptr(), self.phi[1].data_ptr()),
-                       (ctypes.c_void_p * 2)(self.vel[0].data_ptr(), self.vel[1].data_ptr()),
-                       ctypes.c_void_p(self.scratch.data_ptr()),
-                       ctypes.c_size_t(self.scratch.numel()))
+        # phi[1] lies one stride behind phi[0] (indexing would make a tensor)
+        phi, vel, scratch = self.phi, self.vel, self.scratch
+        p, v = phi.data_ptr(), vel.data_ptr()
+        return c_state(_VoidP2(p, p + phi.stride(0) * phi.element_size()),
+                       _VoidP2(v, v + vel.stride(0) * vel.element_size()),
+                       scratch.data_ptr(), scratch.numel())
 
     def report(self, stream=None) -> dict:
         return read_report(self.lat, self, stream)
@@ -345,8 +367,11 @@ class State:
         return self.vel[self.report(stream)["cur"]]
 
 
+_REPORT_KEYS = tuple(k for k, _ in c_report._fields_)
+
+
 def _rep_dict(r: c_report) -> dict:
-    return {k: getattr(r, k) for k, _ in c_report._fields_}
+    return {k: getattr(r, k) for k in _REPORT_KEYS}
 
 
 def init_field(lat: Lattice, seed: Seed, st: State, stream=None):

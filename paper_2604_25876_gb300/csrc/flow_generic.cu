@@ -451,8 +451,9 @@ template <typename T> __global__ void __launch_bounds__(512, 2) k_fixup(FlowPara
 // in pinned host memory and then read over the host link) phi[0] <- src too;
 // without one the interior of phi[0] is not written again.
 // Bound by DRAM: one buffer read and three (with a source four) written.
-// 512^3 FP32, after a copy of the caller's field into phi[0] and with phi[0]
-// rewritten, before: MEASURED
+// load_field of a device tensor, us (with the copy into phi[0] and phi[0]
+// rewritten, before -> now): 128^3 56 -> 35, 256^3 308 -> 231, 512^3 2393 -> 1791
+// (10.7 GB, 6.0 TB/s).
 template <typename T, bool SRC>
 __global__ void __launch_bounds__(256) k_load_field(FlowParams<T> p, const vec4_t<T> *__restrict__ src)
 {
