@@ -23,9 +23,14 @@
 //    warp to be done with a slot (a shared-memory counter) streams the next
 //    plane into it, so the only CTA-wide barriers are at the ends of runs.
 //  * the in-plane values a plane contributes to its own centre two planes
-//    later (13 per site) wait in tensor memory: each warp keeps a 3-slot ring
-//    of them in its TMEM lanes (tcgen05.st / tcgen05.ld), which takes them
-//    off the shared-memory pipe and out of shared memory.
+//    later (12 per site) wait in tensor memory: each warp keeps a ring of them
+//    in its TMEM lanes (tcgen05.st / tcgen05.ld), which takes them off the
+//    shared-memory pipe and out of shared memory.  Three records are in
+//    flight; the ring has five, so that its addresses are constants of the
+//    x-loop, which is unrolled by five.  With three they were computed for
+//    every plane: 270 against 265 us a step at 256^3, 403 against 391 us for
+//    a batch of 16 lattices of 64^3 to 128^3 on 16 x 16 columns.  (The sextic
+//    variant's records are twice as long; its ring stays at three.)
 //  * derivatives are carried without their 1/(12h), 1/(12h^2) factors (the
 //    first-derivative stencil is then 3 instructions per component pair, the
 //    second 4); the factors move into the time step, the mass terms and the
@@ -102,7 +107,7 @@ struct InstDesc {
     // force then comes out as F / B,
     // B = 1/(1728 h^4); B moves into the time step and the mass terms, and
     // the sums are scaled in the finish.
-    float2 dt, dt2;        // dt and 2 dt B
+    float2 dt, dt2;        // dt (1 for the gradient flow, whose update has no velocity) and 2 dt B
     float m2;              // m^2 (potential energy density)
     float bm2;             // m^2 / B (its force term)
     float negK;            // -144 h^2: the quadratic term of the force against the quartic ones
@@ -190,7 +195,7 @@ template <bool SEX> constexpr int rec_cols() { return SEX ? 32 : 16; }
 constexpr int kDzCol = 3 * 32;
 template <bool SEX> constexpr int tmem_cols_per_warp()
 {
-    return SEX ? 128 : 3 * rec_cols<SEX>();  // 3 records in flight (+ the d_z ring)
+    return SEX ? 128 : 5 * rec_cols<SEX>();  // 3 records + the d_z ring; or five records
 }
 template <int NW, bool SEX = false> constexpr uint32_t tmem_cols()
 {
@@ -479,7 +484,7 @@ __device__ __forceinline__ void plane_record(const float4 (*DY)[TZ + 4], const I
 // Euler-Lagrange force of Eq. (3.3) projected on the tangent space, the
 // symplectic update with renormalisation, and the energy, charge and force
 // densities into a32 (valid sites only).
-template <int TY, int TZ, bool POT = false, bool DUMP = false, bool SEX = false>
+template <int TY, int TZ, bool POT = false, bool DUMP = false, bool SEX = false, bool BATCHED = false>
 __device__ __forceinline__ void centre_site(const InstDesc &D, const PlaneVals &M2,
                                             const PlaneVals &M1, const PlaneVals &C,
                                             const PlaneVals &Q1, const PlaneVals &Q2, float2 xc1,
@@ -628,11 +633,15 @@ __device__ __forceinline__ void centre_site(const InstDesc &D, const PlaneVals &
     const float bp = dot(br, ph);
     const P4 Fh = fma(bc(-bp), ph, br);
     const float f2 = 4.f * dot(Fh, Fh);
+    // The gradient flow is the same update from a zero velocity that is not
+    // stored, with dt = 1 in its descriptor: without a branch around it the
+    // step takes 263 us instead of 265 at 256^3.  The sextic and the batched
+    // potentials kernels keep the branch: they are short of registers.
     P4 t, vnew;
-    if (mode == MODE_GRADIENT) {
+    const P4 vo = use_v ? ld4(*vp) : P4{bc(0.f), bc(0.f)};
+    if ((SEX || (BATCHED && POT)) && mode == MODE_GRADIENT) {
         t = fma(dt2, Fh, ph);
     } else {
-        const P4 vo = use_v ? ld4(*vp) : P4{bc(0.f), bc(0.f)};
         vnew = fma(dt2, Fh, vo);
         t = fma(dt, vnew, ph);
     }
@@ -1096,9 +1105,9 @@ __global__ void __launch_bounds__(TY *TZ, 512 / (TY * TZ))
                     const int x = pp - 2;
                     __syncwarp();
                     if (x >= xs)
-                        centre_site<TY, TZ, POT, DUMP, SEX>(D, ring[(k + 1) % 5], ring[(k + 2) % 5], ring[(k + 3) % 5],
+                        centre_site<TY, TZ, POT, DUMP, SEX, BATCHED>(D, ring[(k + 1) % 5], ring[(k + 2) % 5], ring[(k + 3) % 5],
                                             ring[(k + 4) % 5], ring[k], kXm1(), kXm2(),
-                                            twarp + RECC * g3n,
+                                            SEX ? twarp + RECC * g3n : twarp + RECC * ((k + 3) % 5),
                                             make_uint4(twarp + kDzCol + 4 * ((k + 1) % 5),
                                                        twarp + kDzCol + 4 * ((k + 2) % 5),
                                                        twarp + kDzCol + 4 * ((k + 3) % 5),
@@ -1119,7 +1128,8 @@ __global__ void __launch_bounds__(TY *TZ, 512 / (TY * TZ))
                             }
                         }
                     }
-                    plane_record<TY, TZ, SEX>(DY, D, ty, tz, ring[k], dyy, dzz, twarp + RECC * g3);
+                    plane_record<TY, TZ, SEX>(DY, D, ty, tz, ring[k], dyy, dzz,
+                                                SEX ? twarp + RECC * g3 : twarp + RECC * k);
                     if constexpr (SEX) {
                         const float zr[4] = {ring[k].dz.a.x, ring[k].dz.a.y, ring[k].dz.b.x, ring[k].dz.b.y};
                         tmem_st4(twarp + kDzCol + 4 * k, zr);
@@ -1461,7 +1471,7 @@ static bool fill_desc(InstDesc &d, const skyrme_lattice &lat, const skyrme_state
     d.s_b = split(k1 * k1 * k1);
     d.s_e6 = split(k1 * k1 * k1 * k1 * k1 * k1);
     d.s_f = split(B * B);
-    d.dt = make_float2((float)dt, (float)dt);
+    d.dt = pair(mode == MODE_GRADIENT ? 1.0 : dt);
     d.dt2 = pair(2.0 * dt * B);
     const double h3 = lat.h * lat.h * lat.h;
     d.h3_hi = (float)h3;
