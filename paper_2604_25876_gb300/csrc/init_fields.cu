@@ -11,6 +11,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "lattice_sites.cuh"
+#include "packed_f32.cuh"
 #include "skyrme_device.cuh"
 #include "skyrme_internal.h"
 
@@ -144,19 +146,16 @@ constexpr size_t kProfileTableBytes = (size_t)kProfileIntervals * kProfileTerms 
 // First interval: of q = 2^(e - 12), e the exponent of scale^2.
 static int profile_base(double scale) { return (ilogb(scale * scale) - 12 + 1023) * 32; }
 
-__global__ void k_profile_table(double2 *table, int base, double scale)
+// Taylor coefficients, to degree N - 1, of C and S about q (in powers of q' - q).
+template <int N> __device__ __forceinline__ void profile_series(double q, double scale, double (&C)[N], double (&Q)[N])
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= kProfileIntervals) return;
-    constexpr int N = kProfileTerms;
-    const double q = __hiloint2double(((base + i) << 15) | (1 << 14), 0);  // the interval's centre
     // rho to twice the precision, so that exp(-rho) is good to its own rounding
     const double is = 1.0 / scale, is_lo = ::fma(-is, scale, 1.0) * is;
     const double r = sqrt(q), r_lo = ::fma(-r, r, q) / (2.0 * r);
     const double a = r * is, a_lo = ::fma(r, is, -a) + ::fma(r, is_lo, r_lo * is);
     // series in tau = (q' - q) / q: b of sqrt(1 + tau), E of exp(-rho), S and C
     // of sine and cosine of f = pi E, Q of S / r
-    double b[N], E[N], S[N], C[N], Q[N];
+    double b[N], E[N], S[N];
     b[0] = 1.0;
     E[0] = exp(-a);
     E[0] -= E[0] * a_lo;
@@ -188,9 +187,24 @@ __global__ void k_profile_table(double2 *table, int base, double scale)
 #pragma unroll
         for (int j = 1; j <= k; ++j) v -= b[j] * Q[k - j];
         Q[k] = v;
-        table[i * N + k] = make_double2(C[k] * qk, v * qk);
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        C[k] *= qk;
+        Q[k] *= qk;
         qk /= q;
     }
+}
+
+__global__ void k_profile_table(double2 *table, int base, double scale)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= kProfileIntervals) return;
+    constexpr int N = kProfileTerms;
+    double C[N], S[N];
+    profile_series<N>(__hiloint2double(((base + i) << 15) | (1 << 14), 0), scale, C, S);  // the interval's centre
+#pragma unroll
+    for (int k = 0; k < N; ++k) table[i * N + k] = make_double2(C[k], S[k]);
 }
 
 // C and S at q = r^2, directly.
@@ -203,6 +217,57 @@ __device__ __forceinline__ void profile_direct(double q, double scale, double in
     rho = ::fma(::fma(-rho, scale, r), inv_scale, rho);
     sincospi(exp(-rho), &s, &c);
     s *= inv;
+}
+
+// The ansatz at one site in FP64.
+template <bool SYM, bool TAB>
+__device__ __forceinline__ void product_site(const ProductArgs &a, double cx, double cy, double cz, double out[4])
+{
+    // forward product U_1 U_2 ... U_K; the reverse product is
+    // accumulated by left multiplication: U_K ... U_1
+    double fwd[4], rev[4];
+    for (int k = 0; k < a.K; ++k) {
+        const Constituent &c = a.c[k];
+        const double dx = cx - c.pos[0], dy = cy - c.pos[1], dz = cz - c.pos[2];
+        const double q = dx * dx + dy * dy + dz * dz;
+        double cf, sf;
+        const int j = (__double2hiint(q) >> 15) - a.base;
+        if (TAB && j >= 0 && j < kProfileIntervals) {
+            const double2 *t = a.table + j * kProfileTerms;
+            const double d = q - __hiloint2double(((a.base + j) << 15) | (1 << 14), 0);
+            double2 v = __ldg(t + kProfileTerms - 1);
+            cf = v.x, sf = v.y;
+#pragma unroll
+            for (int m = kProfileTerms - 2; m >= 0; --m) {
+                v = __ldg(t + m);
+                cf = ::fma(cf, d, v.x);
+                sf = ::fma(sf, d, v.y);
+            }
+        } else {
+            profile_direct(q, a.scale, a.inv_scale, cf, sf);
+        }
+        const double u[4] = {cf * c.norm, sf * (c.rot[0][0] * dx + c.rot[0][1] * dy + c.rot[0][2] * dz),
+                             sf * (c.rot[1][0] * dx + c.rot[1][1] * dy + c.rot[1][2] * dz),
+                             sf * (c.rot[2][0] * dx + c.rot[2][1] * dy + c.rot[2][2] * dz)};
+        if (k == 0) {
+#pragma unroll
+            for (int m = 0; m < 4; ++m) fwd[m] = rev[m] = u[m];
+        } else {
+            su2_mul(fwd, u, fwd);
+            if (SYM) su2_mul(u, rev, rev);
+        }
+    }
+    if (SYM) {
+        const double t[4] = {fwd[0] + rev[0], fwd[1] + rev[1], fwd[2] + rev[2], fwd[3] + rev[3]};
+        const double n2s = t[0] * t[0] + t[1] * t[1] + t[2] * t[2] + t[3] * t[3];
+        const bool small = n2s < 1e-24;
+        const double rn = rsqrt(n2s);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) out[m] = small ? fwd[m] : t[m] * rn;
+    } else {
+#pragma unroll
+        for (int m = 0; m < 4; ++m) out[m] = fwd[m];
+    }
 }
 
 // The product ansatz over the whole state: the field into both buffers, its
@@ -232,51 +297,7 @@ __global__ void __launch_bounds__(256) k_seed_product(vec4_t<T> *phi0, vec4_t<T>
         double out[4] = {1.0, 0.0, 0.0, 0.0};
         if (interior(x, y, z, n0, n1, n2)) {
             const double cx = coord(x, n0, h), cy = coord(y, n1, h), cz = coord(z, n2, h);
-            // forward product U_1 U_2 ... U_K; the reverse product is
-            // accumulated by left multiplication: U_K ... U_1
-            double fwd[4], rev[4];
-            for (int k = 0; k < a.K; ++k) {
-                const Constituent &c = a.c[k];
-                const double dx = cx - c.pos[0], dy = cy - c.pos[1], dz = cz - c.pos[2];
-                const double q = dx * dx + dy * dy + dz * dz;
-                double cf, sf;
-                const int j = (__double2hiint(q) >> 15) - a.base;
-                if (TAB && j >= 0 && j < kProfileIntervals) {
-                    const double2 *t = a.table + j * kProfileTerms;
-                    const double d = q - __hiloint2double(((a.base + j) << 15) | (1 << 14), 0);
-                    double2 v = __ldg(t + kProfileTerms - 1);
-                    cf = v.x, sf = v.y;
-#pragma unroll
-                    for (int m = kProfileTerms - 2; m >= 0; --m) {
-                        v = __ldg(t + m);
-                        cf = ::fma(cf, d, v.x);
-                        sf = ::fma(sf, d, v.y);
-                    }
-                } else {
-                    profile_direct(q, a.scale, a.inv_scale, cf, sf);
-                }
-                const double u[4] = {cf * c.norm, sf * (c.rot[0][0] * dx + c.rot[0][1] * dy + c.rot[0][2] * dz),
-                                     sf * (c.rot[1][0] * dx + c.rot[1][1] * dy + c.rot[1][2] * dz),
-                                     sf * (c.rot[2][0] * dx + c.rot[2][1] * dy + c.rot[2][2] * dz)};
-                if (k == 0) {
-#pragma unroll
-                    for (int m = 0; m < 4; ++m) fwd[m] = rev[m] = u[m];
-                } else {
-                    su2_mul(fwd, u, fwd);
-                    if (SYM) su2_mul(u, rev, rev);
-                }
-            }
-            if (SYM) {
-                const double t[4] = {fwd[0] + rev[0], fwd[1] + rev[1], fwd[2] + rev[2], fwd[3] + rev[3]};
-                const double n2s = t[0] * t[0] + t[1] * t[1] + t[2] * t[2] + t[3] * t[3];
-                const bool small = n2s < 1e-24;
-                const double rn = rsqrt(n2s);
-#pragma unroll
-                for (int m = 0; m < 4; ++m) out[m] = small ? fwd[m] : t[m] * rn;
-            } else {
-#pragma unroll
-                for (int m = 0; m < 4; ++m) out[m] = fwd[m];
-            }
+            product_site<SYM, TAB>(a, cx, cy, cz, out);
         }
         put<T>(phi0 + s, out);
         put<T>(phi1 + s, out);
@@ -284,6 +305,330 @@ __global__ void __launch_bounds__(256) k_seed_product(vec4_t<T> *phi0, vec4_t<T>
         store4<T>(vel0 + s, zero);
         store4<T>(vel1 + s, zero);
     }
+}
+
+// ---- the ansatz of a large FP32 state, in double-floats
+//
+// The field of an FP32 state is rounded to 24 bits at the end, and the FP32
+// pipe issues 64 times the FP64 pipe's instructions.  k_seed_product_f32
+// evaluates the ansatz in unevaluated sums hi + lo of two floats (error-free
+// products by FMA, Knuth's and Dekker's sums), with a bound on the error beside
+// it, and stores hi where no value within the bound rounds to another float:
+// it is then the rounding of the exact field.  The sites where the bound does
+// not decide (one in 150 with eight constituents), and those where a profile is
+// outside the table, are collected per warp and evaluated in FP64, 32 at a time.
+//
+// Positions are in units of the profile's scale.  A warp takes 32 sites along
+// z; the rotated offsets R_k (x - x_k) of its middle come from FP64 once per
+// warp, a lane's own are off by (lane - 16) R_k e_z h.  The profile comes from
+// a table of Taylor polynomials of degree 6 in q, 256 intervals to an octave
+// (450 KB; the part in use lies in L1), the first three coefficients in
+// double-floats: below 2^-46 of the value for rho < 16, 2^-42 up to 32.
+// U_1 ... U_k and the conjugate of U_k ... U_1 are the two halves of the
+// packed FP32 instructions: the second is the product of the conjugates.
+//
+// Bound by the FP32 pipe (about 85% busy; 400 warp instructions per 32 sites and
+// constituent, three quarters of them FP32, most of those packed).  FP64 and
+// double-float, symmetrised: 256^3 with 8 constituents 17.6 and 2.35 ms, with one
+// 2.07 and 0.53 ms (268 MB written four times: 0.16 ms); 151^3 with 4 constituents
+// 1.84 and 0.33 ms; 128^3 with 64 constituents 17.5 and 3.3 ms.
+constexpr int kPairOctaves = 22, kPairPerOctave = 256;  // q / scale^2 from 2^-12 to 2^10
+constexpr int kPairIntervals = kPairOctaves * kPairPerOctave;
+constexpr int kPairBase = (127 - 12) * kPairPerOctave;
+constexpr int kPairVecs = 5;  // float4 per interval: (C, S) pairs hi, lo of degrees 0 to 2, then 3 to 6
+constexpr size_t kPairTableBytes = (size_t)kPairIntervals * kPairVecs * sizeof(float4);
+// The bounds err[] below: the scalar component's error against 1, the others'
+// against the sum of the constituents' pion sizes.  Over lattice spacings of 0.02
+// to 2 scales and 1 to 64 constituents the largest error met was 0.15 of them.
+constexpr float kPairEps = 0x1p-40f;
+
+__global__ void k_pair_table(float4 *table)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= kPairIntervals) return;
+    constexpr int N = 7;
+    double C[N], S[N];
+    profile_series<N>((double)__int_as_float(((kPairBase + i) << 15) | (1 << 14)), 1.0, C, S);
+    float4 *t = table + i * kPairVecs;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float c = (float)C[k], v = (float)S[k];
+        t[k] = make_float4(c, v, (float)(C[k] - (double)c), (float)(S[k] - (double)v));
+    }
+    t[3] = make_float4((float)C[3], (float)S[3], (float)C[4], (float)S[4]);
+    t[4] = make_float4((float)C[5], (float)S[5], (float)C[6], (float)S[6]);
+}
+
+// -x off the FP32 pipe
+__device__ __forceinline__ float neg(float x) { return __int_as_float(__float_as_int(x) ^ (int)0x80000000); }
+// s + e = a + b exactly
+__device__ __forceinline__ void two_sum(float2 a, float2 b, float2 &s, float2 &e)
+{
+    const float2 m1 = bc(-1.f);
+    s = __fadd2_rn(a, b);
+    const float2 bb = __ffma2_rn(a, m1, s);                                               // s - a
+    e = __fadd2_rn(__ffma2_rn(__ffma2_rn(bb, m1, s), m1, a), __ffma2_rn(bb, m1, b));
+}
+// (ch + cl) + (xh + xl)(d + dl), two quantities; nd = -d
+__device__ __forceinline__ void horner(float2 ch, float2 cl, float2 &xh, float2 &xl, float2 d, float2 nd, float2 dl)
+{
+    const float2 n = __fmul2_rn(xh, nd);
+    float2 e = __ffma2_rn(xh, d, n);
+    e = __ffma2_rn(xl, d, e);
+    e = __ffma2_rn(xh, dl, e);
+    two_sum(ch, __fmul2_rn(xh, d), xh, xl);
+    xl = __fadd2_rn(xl, __fadd2_rn(cl, e));
+}
+// sum_j x_j y_j of pairs of double-floats, n = -y.  The products are added to
+// `shift`, 3 times a power of two above twice their partial sums: each addition
+// then rounds at the same place, and what it drops is exact in two operations.
+struct Pairs4 {
+    float2 h[4], l[4];
+};
+__device__ __forceinline__ void dot_pairs(const float2 (&xh)[4], const float2 (&xl)[4], const float2 (&y)[4],
+                                          const float2 (&ny)[4], const float2 (&nyl)[4], float2 shift, float2 &h,
+                                          float2 &l)
+{
+    float2 p[4], n;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) p[j] = __fmul2_rn(xh[j], y[j]);
+    n = __ffma2_rn(xh[0], ny[0], p[0]);  // minus the product's rounding error
+#pragma unroll
+    for (int j = 1; j < 4; ++j) n = __fadd2_rn(n, __ffma2_rn(xh[j], ny[j], p[j]));
+#pragma unroll
+    for (int j = 0; j < 4; ++j) n = __ffma2_rn(xl[j], ny[j], __ffma2_rn(xh[j], nyl[j], n));
+    const float2 m1 = bc(-1.f);
+    float2 s = shift;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float2 t = __fadd2_rn(s, p[j]);
+        const float2 r = __ffma2_rn(s, m1, t);  // p_j as rounded
+        n = __fadd2_rn(n, __ffma2_rn(p[j], m1, r));
+        s = t;
+    }
+    s = __ffma2_rn(shift, m1, s);
+    h = __ffma2_rn(n, m1, s);
+    l = __ffma2_rn(n, m1, __ffma2_rn(h, m1, s));
+}
+// x y of two quantities' quaternions, y given with its negative
+__device__ __forceinline__ void mul_pairs(Pairs4 &x, const Pairs4 &y, const Pairs4 &n, float2 shift0, float2 shift)
+{
+    Pairs4 r;
+    const auto row = [&](int i, float2 y0, float2 y1, float2 y2, float2 y3, float2 n0, float2 n1, float2 n2, float2 n3,
+                         float2 l0, float2 l1, float2 l2, float2 l3) {
+        const float2 yy[4] = {y0, y1, y2, y3}, nn[4] = {n0, n1, n2, n3}, nl[4] = {l0, l1, l2, l3};
+        dot_pairs(x.h, x.l, yy, nn, nl, i == 0 ? shift0 : shift, r.h[i], r.l[i]);
+    };
+    row(0, y.h[0], n.h[1], n.h[2], n.h[3], n.h[0], y.h[1], y.h[2], y.h[3], n.l[0], y.l[1], y.l[2], y.l[3]);
+    row(1, y.h[1], y.h[0], n.h[3], y.h[2], n.h[1], n.h[0], y.h[3], n.h[2], n.l[1], n.l[0], y.l[3], n.l[2]);
+    row(2, y.h[2], y.h[3], y.h[0], n.h[1], n.h[2], n.h[3], n.h[0], y.h[1], n.l[2], n.l[3], n.l[0], y.l[1]);
+    row(3, y.h[3], n.h[2], y.h[1], y.h[0], n.h[3], y.h[2], n.h[1], n.h[0], n.l[3], y.l[2], n.l[1], n.l[0]);
+    x = r;
+}
+
+// The ansatz at a lane's site: val[] its components hi + lo, err[] bounds on the
+// errors of the scalar component and of the others.  ob[3 k + i]: component i
+// of the rotated offset of constituent k from the warp's middle (hi, lo) and
+// its increment along z (hi, lo); zl: the lane's site from the middle.  False
+// where a profile is outside the table.
+template <bool SYM>
+__device__ __forceinline__ bool product_pairs(const float4 *ob, int K, const float4 *__restrict__ table, float zl,
+                                              float hs, DF (&val)[4], float (&err)[2])
+{
+    Pairs4 x;  // U_1 ... U_k and the conjugate of U_k ... U_1, which is conj(U_1) ... conj(U_k)
+    float P = 0.f;
+    for (int k = 0; k < K; ++k) {
+        float ph[3], pl[3], qh = 0.f, ql = 0.f;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const float4 o = ob[3 * k + i];
+            const float w = __fmul_rn(o.z, zl);
+            const float we = __fmaf_rn(o.w, zl, __fmaf_rn(o.z, zl, -w));
+            two_sum(o.x, w, ph[i], pl[i]);
+            pl[i] = __fadd_rn(pl[i], __fadd_rn(o.y, we));
+            const float t = __fmul_rn(ph[i], ph[i]);
+            const float te = __fmaf_rn(__fadd_rn(pl[i], pl[i]), ph[i], __fmaf_rn(ph[i], ph[i], -t));
+            if (i == 0) {
+                qh = t, ql = te;
+            } else {
+                float e;
+                two_sum(qh, t, qh, e);
+                ql = __fadd_rn(ql, __fadd_rn(e, te));
+            }
+        }
+        const DF q = quick_two_sum(qh, ql);
+        const int bits = __float_as_int(q.hi), j = (bits >> 15) - kPairBase;
+        if ((unsigned)j >= (unsigned)kPairIntervals) return false;
+        const float4 *t = table + j * kPairVecs;
+        const float4 t0 = __ldg(t), t1 = __ldg(t + 1), t2 = __ldg(t + 2), t3 = __ldg(t + 3), t4 = __ldg(t + 4);
+        // q from the interval's centre (the subtraction is exact)
+        const DF dq = quick_two_sum(__fsub_rn(q.hi, __int_as_float((bits & ~0x7fff) | 0x4000)), q.lo);
+        const float2 d = bc(dq.hi), nd = bc(-dq.hi), dl = bc(dq.lo);
+        float2 xh = __ffma2_rn(make_float2(t4.z, t4.w), d, make_float2(t4.x, t4.y));
+        xh = __ffma2_rn(xh, d, make_float2(t3.z, t3.w));
+        xh = __ffma2_rn(xh, d, make_float2(t3.x, t3.y));
+        float2 xl = __ffma2_rn(xh, d, make_float2(t2.z, t2.w));
+        xh = make_float2(t2.x, t2.y);
+        horner(make_float2(t1.x, t1.y), make_float2(t1.z, t1.w), xh, xl, d, nd, dl);
+        horner(make_float2(t0.x, t0.y), make_float2(t0.z, t0.w), xh, xl, d, nd, dl);
+        // U_k and its conjugate
+        Pairs4 y, n;
+        y.h[0] = bc(xh.x), y.l[0] = bc(xl.x);
+        n.h[0] = bc(neg(xh.x)), n.l[0] = bc(neg(xl.x));
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const float u = __fmul_rn(xh.y, ph[i]);
+            const float ul = __fmaf_rn(xl.y, ph[i], __fmaf_rn(xh.y, pl[i], __fmaf_rn(xh.y, ph[i], -u)));
+            y.h[i + 1] = make_float2(u, neg(u)), n.h[i + 1] = make_float2(neg(u), u);
+            y.l[i + 1] = make_float2(ul, neg(ul)), n.l[i + 1] = make_float2(neg(ul), ul);
+            P = __fadd_rn(P, fabsf(u));
+        }
+        P = __fmaf_rn(0.25f * hs, xh.y, P);  // the offsets' own rounding (they reach 16 sites from the lane's)
+        if (k == 0) {
+            x = y;
+        } else {
+            // the vector components' partial sums stay below 2 P, the scalar's below 1
+            const float big = __int_as_float(((__float_as_int(P) & 0x7f800000) + (3 << 23)) | 0x400000);
+            mul_pairs(x, y, n, bc(3.f), bc(big));
+        }
+    }
+    const float eps = kPairEps * __fmaf_rn(4.f, hs, 1.f), eps0 = eps * (1.f + (float)K),
+                eps1 = eps * __fmaf_rn(0.0625f, (float)K, 1.f);
+    if (!SYM) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) val[i] = quick_two_sum(x.h[i].x, x.l[i].x);
+        err[0] = eps0, err[1] = eps1 * P;
+        return true;
+    }
+    // t = U_1 ... U_K + U_K ... U_1, divided by its norm
+    DF t[4], q = {0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float sg = i == 0 ? 1.f : -1.f;
+        float s, e;
+        two_sum(x.h[i].x, sg * x.h[i].y, s, e);
+        t[i] = quick_two_sum(s, __fadd_rn(e, __fmaf_rn(sg, x.l[i].y, x.l[i].x)));
+        q = df_add(q, df_mul(t[i], t[i]));
+    }
+    if (!(q.hi > 0x1p-20f)) return false;
+    // 1 / sqrt(q): y0 and one step, q y0^2 = 1 - g
+    const float y0 = rsqrtf(q.hi), a = __fmul_rn(y0, y0), ae = __fmaf_rn(y0, y0, -a);
+    const float b = __fmul_rn(q.hi, a);
+    const float be = __fmaf_rn(q.lo, a, __fmaf_rn(q.hi, ae, __fmaf_rn(q.hi, a, -b)));
+    const float g = __fsub_rn(__fsub_rn(1.f, b), be);
+    const DF y = {y0, __fmul_rn(__fmul_rn(y0, g), __fmaf_rn(0.375f, g, 0.5f))};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) val[i] = df_mul(t[i], y);
+    const float y2 = 4.f * (y0 * y0);
+    err[0] = eps0 * y2, err[1] = eps1 * P * y2;
+    return true;
+}
+
+// An integer as a double, by one FP64 addition.
+__device__ __forceinline__ double to_double(int i)
+{
+    return __hiloint2double(0x43300000, i ^ (int)0x80000000) - (0x1p52 + 0x1p31);
+}
+
+// The sites the bound left open, in FP64.
+template <bool SYM>
+__device__ __noinline__ void product_open(const ProductArgs &a, float4 *phi0, float4 *phi1, unsigned s, int n0, int n1,
+                                          int n2, double h)
+{
+    const unsigned row = s / (unsigned)n2;
+    const int z = (int)(s - row * (unsigned)n2), y = (int)(row % (unsigned)n1), x = (int)(row / (unsigned)n1);
+    double out[4];
+    product_site<SYM, false>(a, coord(x, n0, h), coord(y, n1, h), coord(z, n2, h), out);
+    put<float>(phi0 + s, out);
+    put<float>(phi1 + s, out);
+}
+
+constexpr int kPairWarps = 8;
+template <bool SYM>
+__global__ void __launch_bounds__(32 * kPairWarps, 2)
+    k_seed_product_f32(float4 *phi0, float4 *phi1, float4 *vel0, float4 *vel1, int n0, int n1, int n2, double h,
+                       const __grid_constant__ ProductArgs a, const float4 *table, unsigned table_sites)
+{
+    __shared__ double s_row[3 * kMaxConstituents][4];  // change per half step in x, y, z; offset of the centre
+    __shared__ float2 s_dz[3 * kMaxConstituents];      // change per step in z
+    __shared__ float4 s_ob[kPairWarps][3 * kMaxConstituents];
+    __shared__ unsigned s_open[kPairWarps][64];
+    __shared__ int s_left[kPairWarps];
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, K3 = 3 * a.K;
+    const double hs = h * a.inv_scale;
+    for (int i = threadIdx.x; i < K3; i += blockDim.x) {
+        const Constituent &c = a.c[i / 3];
+        const double *r = c.rot[i % 3];
+        for (int j = 0; j < 3; ++j) s_row[i][j] = 0.5 * (r[j] * hs);
+        const double dz = r[2] * hs;
+        s_dz[i] = make_float2((float)dz, (float)(dz - (double)(float)dz));
+        s_row[i][3] = -(r[0] * c.pos[0] + r[1] * c.pos[1] + r[2] * c.pos[2]) * a.inv_scale;
+    }
+    __syncthreads();
+    const unsigned segs = ((unsigned)n2 + 31) / 32, items = (unsigned)n0 * n1 * segs;
+    int open = 0;
+    for (unsigned it = blockIdx.x * kPairWarps + warp; it < items; it += gridDim.x * kPairWarps) {
+        // (the segments are rotated by a hash of the row, or a warp could get the same one,
+        // with more or fewer open sites than the others', every time)
+        const unsigned row = it / segs;
+        const int zc = (int)((it - row * segs + (row * 0x9E3779B9u >> 16)) % segs) * 32 + 16, z = zc - 16 + lane;
+        const int y = (int)(row % (unsigned)n1), x = (int)(row / (unsigned)n1);
+        const unsigned s = row * (unsigned)n2 + z;
+        float4 out = make_float4(1.f, 0.f, 0.f, 0.f);
+        bool sure = true;
+        if (x >= 2 && x <= n0 - 3 && y >= 2 && y <= n1 - 3) {
+            const double xi = to_double(2 * x - (n0 - 1)), yi = to_double(2 * y - (n1 - 1)),
+                         zi = to_double(2 * zc - (n2 - 1));
+            for (int i = lane; i < K3; i += 32) {
+                const double *r = s_row[i], o = ::fma(r[0], xi, ::fma(r[1], yi, ::fma(r[2], zi, r[3])));
+                const float oh = (float)o;
+                const float2 dz = s_dz[i];
+                s_ob[warp][i] = make_float4(oh, (float)(o - widen(oh)), dz.x, dz.y);
+            }
+            __syncwarp();
+            if (z >= 2 && z <= n2 - 3) {
+                DF v[4];
+                float err[2];
+                sure = product_pairs<SYM>(s_ob[warp], a.K, table, (float)(lane - 16), (float)hs, v, err);
+                if (sure) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float e = err[i > 0];
+                        sure = sure && __fadd_rn(v[i].hi, __fadd_rn(v[i].lo, e)) == v[i].hi &&
+                               __fadd_rn(v[i].hi, __fsub_rn(v[i].lo, e)) == v[i].hi;
+                    }
+                    out = make_float4(v[0].hi, v[1].hi, v[2].hi, v[3].hi);
+                }
+            }
+            __syncwarp();
+        }
+        if (z < n2) {
+            const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (sure) {
+                phi0[s] = out;
+                phi1[s] = out;
+            }
+            vel0[s] = zero;
+            if (s >= table_sites) vel1[s] = zero;  // (the table is in its first sites)
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, !sure);
+        if (m) {
+            if (!sure) s_open[warp][open + __popc(m & ((1u << lane) - 1))] = s;
+            open += __popc(m);
+            __syncwarp();
+            if (open >= 32) {
+                open -= 32;
+                product_open<SYM>(a, phi0, phi1, s_open[warp][open + lane], n0, n1, n2, h);
+                __syncwarp();
+            }
+        }
+    }
+    // the sites left over, packed over the block's warps
+    if (lane == 0) s_left[warp] = open;
+    __syncthreads();
+    int i = threadIdx.x, w = 0;
+    while (w < kPairWarps && i >= s_left[w]) i -= s_left[w++];
+    if (w < kPairWarps) product_open<SYM>(a, phi0, phi1, s_open[w][i], n0, n1, n2, h);
 }
 
 // ------------------------------------------------------------------ noise
@@ -422,6 +767,44 @@ static int grid_for(size_t total)
     return (int)(b < 1 ? 1 : b);
 }
 
+// Whether the double-float kernel takes the ansatz: unit orientations, rows that
+// fill a warp, 32-bit indices, offsets small enough for their rounding, and a
+// lattice that lies largely inside the table (32 scales from a constituent):
+// outside, the attempt costs 7% on top of the FP64 evaluation.  At 128^3 with 4
+// constituents, FP64 and double-float: 1.69 and 1.82 ms with nearly every site
+// outside, 1.73 and 1.74 ms with a box of +-64 scales (the estimate is then 0.08).
+static bool pairs_apply(const skyrme_lattice &lat, const ProductArgs &pa)
+{
+    const double total = (double)lat.n[0] * lat.n[1] * lat.n[2];
+    if (lat.n[2] < 24 || total >= 4.2e9 || total * sizeof(float4) < (double)kPairTableBytes) return false;
+    double inside = 1.0;
+    for (int j = 0; j < 3; ++j) {
+        double reach = 0.0;
+        for (int k = 0; k < pa.K; ++k) reach = fmax(reach, fabs(pa.c[k].pos[j]));
+        reach = (reach + 0.5 * lat.n[j] * lat.h) * pa.inv_scale;
+        if (!(reach <= 256.0)) return false;
+        inside *= fmin(1.0, 28.0 / reach);
+    }
+    for (int k = 0; k < pa.K; ++k)
+        if (!(fabs(pa.c[k].norm - 1.0) <= 0x1p-48)) return false;
+    return inside >= 0.3;
+}
+
+static cudaError_t launch_product_f32(const skyrme_lattice &lat, const ProductArgs &pa, bool sym, const FlowArgs &a,
+                                      cudaStream_t s)
+{
+    // the table lies in the first sites of the second velocity buffer, which
+    // are zeroed afterwards
+    float4 *phi0 = static_cast<float4 *>(a.phi[0]), *phi1 = static_cast<float4 *>(a.phi[1]);
+    float4 *v0 = static_cast<float4 *>(a.vel[0]), *v1 = static_cast<float4 *>(a.vel[1]);
+    k_pair_table<<<(kPairIntervals + 31) / 32, 32, 0, s>>>(v1);
+    auto kernel = sym ? k_seed_product_f32<true> : k_seed_product_f32<false>;
+    kernel<<<2 * 152, 32 * kPairWarps, 0, s>>>(phi0, phi1, v0, v1, lat.n[0], lat.n[1], lat.n[2], lat.h, pa, v1,
+                                               (unsigned)(kPairTableBytes / sizeof(float4)));
+    const cudaError_t e = cudaMemsetAsync(v1, 0, kPairTableBytes, s);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 template <typename T>
 static cudaError_t seed_impl(const skyrme_lattice &lat, const skyrme_seed &sd, const FlowArgs &a,
                              size_t scratch_bytes, cudaStream_t s)
@@ -442,18 +825,8 @@ static cudaError_t seed_impl(const skyrme_lattice &lat, const skyrme_seed &sd, c
         pa.K = sd.B;
         pa.scale = sd.profile_scale;
         pa.inv_scale = 1.0 / sd.profile_scale;
-        // The table costs a launch of 26 us and saves 30 instructions per site
-        // and constituent (48 us per million of them); it needs the scratch
-        // behind the control block and an ordinary scale.
         pa.table = nullptr;
         pa.base = 0;
-        if ((double)total * sd.B >= 1e6 && scratch_bytes >= kProfileTableBytes &&
-            sd.profile_scale > 1e-100 && sd.profile_scale < 1e100) {
-            pa.base = profile_base(sd.profile_scale);
-            double2 *table = reinterpret_cast<double2 *>(a.step_parts);
-            k_profile_table<<<(kProfileIntervals + 31) / 32, 32, 0, s>>>(table, pa.base, pa.scale);
-            pa.table = table;
-        }
         for (int k = 0; k < sd.B; ++k) {
             Constituent &c = pa.c[k];
             const double *q = sd.quaternions + 4 * k;
@@ -468,6 +841,20 @@ static cudaError_t seed_impl(const skyrme_lattice &lat, const skyrme_seed &sd, c
             }
             su2_mul(A, Ad, r);
             c.norm = r[0];
+        }
+        // The double-float kernel takes 60 us at least (its table, the FP64
+        // remainder): 64^3 with one constituent 64 us against 79, 32^3 with eight
+        // 91 against 93, 50^3 with one 60 against 60.
+        const double work = (double)total * sd.B;
+        if (sizeof(T) == 4 && work >= 2.5e5 && pairs_apply(lat, pa)) return launch_product_f32(lat, pa, sd.symmetrise, a, s);
+        // The table costs a launch of 26 us and saves 30 instructions per site
+        // and constituent (48 us per million of them); it needs the scratch
+        // behind the control block and an ordinary scale.
+        if (work >= 1e6 && scratch_bytes >= kProfileTableBytes && sd.profile_scale > 1e-100 && sd.profile_scale < 1e100) {
+            pa.base = profile_base(sd.profile_scale);
+            double2 *table = reinterpret_cast<double2 *>(a.step_parts);
+            k_profile_table<<<(kProfileIntervals + 31) / 32, 32, 0, s>>>(table, pa.base, pa.scale);
+            pa.table = table;
         }
         vec4_t<T> *phi1 = static_cast<vec4_t<T> *>(a.phi[1]);
         vec4_t<T> *v0 = static_cast<vec4_t<T> *>(a.vel[0]), *v1 = static_cast<vec4_t<T> *>(a.vel[1]);

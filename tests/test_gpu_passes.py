@@ -166,6 +166,37 @@ def test_product_seed_matches_oracle(n, h, K, scale, prec, sym):
     assert sk.read_report(lat, st)["steps"] == 0
 
 
+# the double-float kernel: rows of 24 sites, of one and a bit of a warp, a
+# constituent on a site, radii on both sides of the table's ends (rho = 1/64
+# and 32), many constituents, a coarse and a fine lattice
+@pytest.mark.parametrize("n,h,K,scale", [((64, 64, 64), 0.15, 1, 1.0), ((47, 51, 24), 0.2, 8, 1.0),
+                                         ((41, 60, 33), 0.02, 4, 1.0), ((60, 63, 95), 0.3, 2, 0.4),
+                                         ((60, 40, 65), 1.0, 3, 2.5), ((28, 33, 35), 0.25, 64, 0.7)])
+@pytest.mark.parametrize("sym", [True, False])
+def test_large_fp32_product_seed_is_the_rounded_fp64_seed(n, h, K, scale, sym):
+    rng = np.random.default_rng(K)
+    pos = rng.uniform(-1.0, 1.0, size=(K, 3)) * min(2.0, 0.3 * h * min(n))
+    pos[0] = [(n[a] // 2 - 0.5 * (n[a] - 1)) * h for a in range(3)]
+    q = rng.normal(size=(K, 4))
+    q /= np.linalg.norm(q, axis=1, keepdims=True)
+    phi = {}
+    for prec in (32, 64):
+        lat = sk.Lattice(n, h, 1.0, prec)
+        st = sk.State(lat, DEV)
+        st.vel.fill_(3.0)
+        sk.init_field(lat, sk.Seed.product(pos, q, scale, sym), st)
+        assert torch.equal(st.phi[0], st.phi[1]) and not st.vel.any().item()
+        phi[prec] = st.phi[0].cpu()
+    # both are within 1e-14 of the exact value (K = 64), so their roundings differ
+    # only where it lies that close to the middle of two floats: 1e-14 / 6e-8 of
+    # the components of size one (and as rarely of the others, whose errors
+    # shrink with them), 0.2 of 1e6; then by one ulp
+    ref = phi[64].float()
+    off = phi[32] != ref
+    assert int(off.sum()) <= 4
+    assert torch.all((phi[32] - ref).abs()[off] <= 1.3e-7 * ref.abs()[off])
+
+
 # the FP64 step's columns (2 x 16 or 4 x 8), runs and shares: lattices of fewer
 # units than warps, runs that cross columns, both column shapes, long runs
 @pytest.mark.parametrize("n", SIZES + [(33, 48, 48), (200, 14, 18)])
