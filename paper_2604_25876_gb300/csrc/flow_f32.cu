@@ -1850,7 +1850,11 @@ cudaError_t launch_iterations_f32_fast(const skyrme_lattice &lat, const FlowArgs
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = fused ? 1 : 0;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = fused ? 1 : 0;
+    // the next step's CTAs start as this one's leave (its prologue runs before
+    // it waits for this launch to end): Newton flow 12.4 -> 11.8 us a step at
+    // 24 x 26 x 28 and 16.4 -> 15.7 at 64^3 in a graph, 14.8 -> 13.0 and 18.9 -> 16.9
+    // on a stream
+    attr[1].val.programmaticStreamSerializationAllowed = a.slab_rec ? 0 : 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(16 * 32);

@@ -26,8 +26,9 @@
 //  * Units per warp decide the time of a small lattice, so the launch takes 8,
 //    6 or 4 warps per SM, whichever leaves the busiest SM less to do
 //    (plan_warps).
-//  * Consecutive steps are programmatic dependents: a step's CTAs start as the
-//    last step's leave, and wait for it before they read anything it wrote.
+//  * Consecutive steps are programmatic dependents (with 8 and 6 warps per CTA):
+//    a step's CTAs start as the last step's leave, and wait for it before they
+//    read anything it wrote.
 //  * Measured (us per iteration, tile kernel and fix-up launch before -> now):
 //    48^3 103.6 -> 78.5, 64^3 187 -> 159, 128^3 1392 -> 1190 (1.60 G
 //    site-updates/s, 341 instructions per site at the measured FP64 FMA rate),
@@ -574,11 +575,14 @@ template <bool EXT, int TZ> static cudaError_t launch_shape(F64Params &p, int sm
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = p.fuse_fix;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = p.fuse_fix;
+    // The next step's CTAs start as this one's leave only where one fits on an
+    // SM: with 4 warps two fit, and a graph then packs some SMs with two of the
+    // next step's (48^3: 127 us a step instead of 74).
+    attr[1].val.programmaticStreamSerializationAllowed =
+        !p.slab_rec && 2 * (sizeof(StepSmem64) + warps * sizeof(WarpSmem<TZ>)) > 228 * 1024;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((used + warps - 1) / warps));
     cfg.blockDim = dim3(32 * warps);
-    // (with 4 warps, the next step's CTAs fit beside this one's)
     cfg.dynamicSmemBytes = sizeof(StepSmem64) + warps * sizeof(WarpSmem<TZ>);
     cfg.stream = s;
     cfg.attrs = attr;
