@@ -315,7 +315,8 @@ static skyrme_status launch_iterations(const skyrme_lattice &lat, const FlowArgs
                                        cudaStream_t s)
 {
     // FP32: the streaming kernel (the standard model, the Section 7.8
-    // potentials, the sextic term); FP64: the tile kernels
+    // potentials, the sextic term); FP64: its own; FP32 without a tensor-map
+    // encoder: the tile kernel and the fix-up
     if (fp32_streaming(lat)) {
         CK(launch_iterations_f32_fast(lat, a, nsteps, s), "step and fix-up kernels (fp32)");
         return SKYRME_OK;
@@ -332,12 +333,11 @@ static skyrme_status launch_iterations(const skyrme_lattice &lat, const FlowArgs
 
 
 // skyrme_flow_step's iterations.  A stream launch costs the GPU about 2.5 us
-// and a kernel node of a graph about 0.8 us, and every iteration is two
-// launches, so a long call captures kGraphChunk iterations once, on a stream
-// of its own, and replays that graph on the caller's stream; the graph and
-// the stream are released before the call returns (a graph still running is
-// freed when it completes).  Short calls, and calls on a stream that is
-// being captured, launch directly.
+// and a kernel node of a graph about 0.8 us, so a long call captures
+// kGraphChunk iterations once, on a stream of its own, and replays that graph
+// on the caller's stream; the graph and the stream are released before the
+// call returns (a graph still running is freed when it completes).  Short
+// calls, and calls on a stream that is being captured, launch directly.
 constexpr int kGraphChunk = 128;
 
 static skyrme_status run_iterations(const skyrme_lattice &lat, const FlowArgs &a, int nsteps,

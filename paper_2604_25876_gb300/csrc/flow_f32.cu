@@ -1,7 +1,7 @@
 // flow_f32.cu -- FP32 streaming step kernel of the arrested Newton flow, for
 // one lattice or a batch of independent lattices of uneven sizes.
 //
-// Same iteration as the tile kernel (Section 3: 4th-order first, second and
+// One iteration (Section 3: 4th-order first, second and
 // mixed derivatives, Euler-Lagrange gradient, tangent projection of
 // Eq. "Newton_flow", v += dt F, phi = normalise(phi + dt v); Section 2.1
 // densities), organised for GB300:
@@ -107,7 +107,9 @@ struct InstDesc {
     // force then comes out as F / B,
     // B = 1/(1728 h^4); B moves into the time step and the mass terms, and
     // the sums are scaled in the finish.
-    float2 dt, dt2;        // dt (1 for the gradient flow, whose update has no velocity) and 2 dt B
+    // v' = v + dt2 F/2B, phi' = phi + dt v': dt2 = 2 dt B; the gradient flow is
+    // the same update with v = 0, dt2 = 1 and 2 dt B in dt
+    float2 dt, dt2;
     float m2;              // m^2 (potential energy density)
     float bm2;             // m^2 / B (its force term)
     float negK;            // -144 h^2: the quadratic term of the force against the quartic ones
@@ -629,18 +631,19 @@ __device__ __forceinline__ void centre_site(const InstDesc &D, const PlaneVals &
         e6 = D.c6 * Dd * Dd;
     }
 
-    // F = -G + (G.phi) phi = 2 B (br - (br.phi) phi); dt2 = 2 dt B
+    // F = -G + (G.phi) phi = 2 B (br - (br.phi) phi)
     const float bp = dot(br, ph);
     const P4 Fh = fma(bc(-bp), ph, br);
     const float f2 = 4.f * dot(Fh, Fh);
-    // The gradient flow is the same update from a zero velocity that is not
-    // stored, with dt = 1 in its descriptor: without a branch around it the
-    // step takes 263 us instead of 265 at 256^3.  The sextic and the batched
-    // potentials kernels keep the branch: they are short of registers.
+    // The gradient flow is the same update from a zero velocity, which is not
+    // stored: v' is then F itself and its time step is in dt.  Without a branch
+    // around it the step takes 263 us instead of 265 at 256^3.  The sextic and
+    // the batched potentials kernels keep the branch: they are short of
+    // registers.
     P4 t, vnew;
     const P4 vo = use_v ? ld4(*vp) : P4{bc(0.f), bc(0.f)};
     if ((SEX || (BATCHED && POT)) && mode == MODE_GRADIENT) {
-        t = fma(dt2, Fh, ph);
+        t = fma(dt, Fh, ph);
     } else {
         vnew = fma(dt2, Fh, vo);
         t = fma(dt, vnew, ph);
@@ -1471,8 +1474,8 @@ static bool fill_desc(InstDesc &d, const skyrme_lattice &lat, const skyrme_state
     d.s_b = split(k1 * k1 * k1);
     d.s_e6 = split(k1 * k1 * k1 * k1 * k1 * k1);
     d.s_f = split(B * B);
-    d.dt = pair(mode == MODE_GRADIENT ? 1.0 : dt);
-    d.dt2 = pair(2.0 * dt * B);
+    d.dt = pair(mode == MODE_GRADIENT ? 2.0 * dt * B : dt);
+    d.dt2 = pair(mode == MODE_GRADIENT ? 1.0 : 2.0 * dt * B);
     const double h3 = lat.h * lat.h * lat.h;
     d.h3_hi = (float)h3;
     d.h3_lo = (float)(h3 - (double)d.h3_hi);

@@ -1,4 +1,5 @@
-// flow_f64.cu -- the FP64 step of the arrested Newton flow (Section 3: 4th-order
+// flow_f64.cu -- the FP64 step of the Newton and arrested Newton flows (gradient
+// flows run on the tile kernel of flow_generic.cu) (Section 3: 4th-order
 // first, second and mixed derivatives, Euler-Lagrange gradient, tangent
 // projection of Eq. "Newton_flow", v += dt F, phi = normalise(phi + dt v);
 // Section 2.1 and 7.8 densities).
@@ -259,7 +260,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_step_f64(const __grid_con
     const dvec4 *__restrict__ vin = cur ? p.vel[1] : p.vel[0];
     dvec4 *__restrict__ phi_out = cur ? p.phi[0] : p.phi[1];
     dvec4 *__restrict__ vel_out = cur ? p.vel[0] : p.vel[1];
-    const bool use_v = p.mode != MODE_GRADIENT && !pred;
+    const bool use_v = !pred;
     const size_t sx = (size_t)p.n1 * p.n2;
     // this warp's units, a contiguous range
     const int wid = blockIdx.x * warps + warp, u0 = p.start[wid], u1 = p.start[wid + 1];
@@ -353,20 +354,14 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_step_f64(const __grid_con
             first(M[2], lds(&ws.uy[s0][ly][lz]), lds(&ws.uy[s0][ly][lz + 1]), lds(&ws.uy[s0][ly][lz + 3]),
                   lds(&ws.uy[s0][ly][lz + 4]));
             step_site<EXT>(p, ph, u, N, M, F, dens);
-            double t[4];
-            if (p.mode == MODE_GRADIENT) {
-#pragma unroll
-                for (int A = 0; A < 4; ++A) t[A] = ::fma(p.dt2, F[A], ph[A]);
-            } else {
-                v = dvec4{::fma(p.dt2, F[0], v.x), ::fma(p.dt2, F[1], v.y), ::fma(p.dt2, F[2], v.z),
-                          ::fma(p.dt2, F[3], v.w)};
-                t[0] = ::fma(p.dt, v.x, ph[0]), t[1] = ::fma(p.dt, v.y, ph[1]);
-                t[2] = ::fma(p.dt, v.z, ph[2]), t[3] = ::fma(p.dt, v.w, ph[3]);
-            }
+            v = dvec4{::fma(p.dt2, F[0], v.x), ::fma(p.dt2, F[1], v.y), ::fma(p.dt2, F[2], v.z),
+                      ::fma(p.dt2, F[3], v.w)};
+            const double t[4] = {::fma(p.dt, v.x, ph[0]), ::fma(p.dt, v.y, ph[1]), ::fma(p.dt, v.z, ph[2]),
+                                 ::fma(p.dt, v.w, ph[3])};
             const double rn = rsqrt(dot4(t, t));  // within an ulp of 1/sqrt, without its division
             if (valid) {
                 const size_t site = (size_t)x * sx + col_site;
-                if (p.mode != MODE_GRADIENT) store4<double>(vel_out + site, v);
+                store4<double>(vel_out + site, v);
                 store4<double>(phi_out + site, dvec4{t[0] * rn, t[1] * rn, t[2] * rn, t[3] * rn});
                 const double f2 = dot4(F, F);
 #pragma unroll

@@ -1,20 +1,23 @@
-// flow_generic.cu -- tile-staged kernels of the arrested Newton flow in either
-// precision: the fused step (derivatives + Euler-Lagrange gradient + tangent
-// projection + velocity/field update + renormalisation + energy sums), the
-// speculative-arrest fix-up and the per-site force dump.
+// flow_generic.cu -- tile-staged kernels of the arrested Newton flow: the
+// per-site force dump in either precision, and the fused step (derivatives +
+// Euler-Lagrange gradient + tangent projection + velocity/field update +
+// renormalisation + energy sums) of FP64 gradient flows and of FP32 fields
+// where the driver has no tensor-map encoder; also the speculative-arrest
+// fix-up and the field load.
 //
 // One CTA owns a TX x TY x TZ block of interior sites and stages the field
 // with a 2-site halo in shared memory (Section 3: stencil radius 2).  The
-// FP64 path is bound by the FP64 pipe, so this straightforward staging is its
-// production kernel; FP32 has a dedicated streaming kernel elsewhere.
+// other flows' kernels are elsewhere: the streaming steps of FP32
+// (flow_f32.cu) and FP64 (flow_f64.cu) fields.
 //
 // Arrest without a host round trip: the energy E_n of phi_n is only known
 // after every CTA has finished, but the update needs to know whether v_n is
 // zeroed.  Each step therefore applies the decision predicted from the
 // previous iteration (ctrl.pred); the last CTA compares E_n with E_{n-1},
 // and when the prediction was wrong it sets ctrl.fix = +-1 so that the
-// pointwise fix-up kernel rewrites v_{n+1} = v' -+ v_n and
-// phi_{n+1} = normalise(phi_n + dt v_{n+1}) from the untouched old buffers.
+// pointwise fix-up (k_fixup, or the streaming steps' own correction) rewrites
+// v_{n+1} = v' -+ v_n and phi_{n+1} = normalise(phi_n + dt v_{n+1}) from the
+// untouched old buffers.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -259,8 +262,8 @@ __device__ __forceinline__ void reduce_and_finish(const FlowParams<T> &p, double
 
 // Resident 256-thread CTAs per SM the register allocation is sized for:
 // three for FP32 (24 warps to hide the latency of the tile loads), two for the
-// standard FP64 kernels, one for the extended FP64 kernels (bound by the FP64
-// pipe either way).
+// standard FP64 kernels, one for the extended ones (bound by the FP64 pipe
+// either way).
 template <typename T, bool EXT>
 constexpr int kTileMinBlocks = sizeof(T) == 4 ? 3 : (EXT ? 1 : 2);
 
@@ -649,6 +652,13 @@ static cudaError_t launch_tile(const skyrme_lattice &lat, const FlowParams<T> &p
 
 cudaError_t launch_step(const skyrme_lattice &lat, const FlowArgs &a, cudaStream_t s)
 {
+    // The gradient flow's explicit step is unstable on steep seeds at the time
+    // steps the other modes take, and then multiplies a rounding difference by
+    // up to 10^9 in 20 steps (a fifth of a sample of 40 FP64 gradient flows): it
+    // keeps the tile kernel and its roundings.  It would gain what the other
+    // modes do (48^3 95 -> 73 us a step).
+    if (lat.precision == 64 && a.mode == MODE_GRADIENT)
+        return launch_tile<double, 0>(lat, make_params<double>(a, a.step_parts), nullptr, nullptr, s);
     if (lat.precision == 64) return launch_step_f64(lat, a, s);
     return launch_tile<float, 0>(lat, make_params<float>(a, a.step_parts), nullptr, nullptr, s);
 }
