@@ -321,6 +321,10 @@ static skyrme_status launch_iterations(const skyrme_lattice &lat, const FlowArgs
         CK(launch_iterations_f32_fast(lat, a, nsteps, s), "step and fix-up kernels (fp32)");
         return SKYRME_OK;
     }
+    if (lat.precision == 64 && a.mode != SKYRME_GRADIENT) {
+        CK(launch_steps_f64(lat, a, nsteps, s), "step kernel (fp64)");
+        return SKYRME_OK;
+    }
     for (int k = 0; k < nsteps; ++k) {
         CK(launch_step(lat, a, s), "step kernel");
         // the FP64 step corrects its own sites; an x-slab's fix-up follows the

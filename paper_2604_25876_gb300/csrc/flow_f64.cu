@@ -27,13 +27,18 @@
 //  * Units per warp decide the time of a small lattice, so the launch takes 8,
 //    6 or 4 warps per SM, whichever leaves the busiest SM less to do
 //    (plan_warps).
-//  * Consecutive steps are programmatic dependents (with 8 and 6 warps per CTA):
-//    a step's CTAs start as the last step's leave, and wait for it before they
-//    read anything it wrote.
+//  * A launch runs several steps of a small lattice (kLaunchSites): every CTA
+//    waits for the decision and goes on to the next step, over one more barrier
+//    when sites were corrected.  One step per launch and now, us per step in a
+//    graph and on a stream: 24 x 26 x 28 26.9 and 29.2 -> 25.7 and 26.0, 48^3
+//    73.7 and 76.3 -> 72.5 and 73.0, 90 x 75 x 83 326 and 329 -> 325 and 325.
+//  * Consecutive launches are programmatic dependents (with 8 and 6 warps per
+//    CTA): a launch's CTAs start as the last one's leave, and wait for it before
+//    they read anything it wrote.
 //  * Measured (us per iteration, tile kernel and fix-up launch before -> now):
-//    48^3 103.6 -> 78.5, 64^3 187 -> 159, 128^3 1392 -> 1190 (1.60 G
-//    site-updates/s, 341 instructions per site at the measured FP64 FMA rate),
-//    90 x 75 x 83 lightly bound 409 -> 337, 72 x 80 x 100 sextic 520 -> 429.
+//    48^3 103.6 -> 73, 64^3 187 -> 153, 128^3 1392 -> 1166 (1.63 G
+//    site-updates/s, 334 instructions per site at the measured FP64 FMA rate),
+//    90 x 75 x 83 lightly bound 409 -> 326, 72 x 80 x 100 sextic 520 -> 429.
 //  * The arrest decision falls in the last CTA to finish; the launch is
 //    cooperative, and every warp corrects its own sites when the decision that
 //    the step ran with was wrong (flow_generic.cu has the scheme).
@@ -52,6 +57,7 @@ namespace skyrme {
 constexpr int kMaxWarps = 8;    // per CTA, one CTA per SM
 constexpr int kMaxShare = 160 * kMaxWarps;  // warps of a launch
 constexpr int kPlaneSlots = 4;  // planes x .. x + 2 of the centre, and the next one arriving
+constexpr double kLaunchSites = 1 << 22;  // site updates of a launch of several steps
 constexpr int kSums64 = 8;      // e2, e4, potential, det, |F|^2, max |F|^2, e6, (unused)
 
 struct F64Params {
@@ -64,6 +70,7 @@ struct F64Params {
     int nix, nzt;      // interior planes, columns along z
     long long units;   // columns * planes
     int mode, fuse_fix;
+    int steps;         // of this launch
     double dt, dt2;    // dt, and 2 dt B
     double K144;       // 144 h^2
     double bm2, bmy2, bmz2, bmw2;  // squared masses / B
@@ -92,6 +99,12 @@ struct __align__(128) StepSmem64 {
 };
 
 __device__ __forceinline__ dvec4 lds(const dvec4 *p) { return load4<double>(p); }
+// A site from L2: L1 may hold what an earlier step of the launch read there
+__device__ __forceinline__ dvec4 ldcg4(const dvec4 *p)
+{
+    const double2 *q = reinterpret_cast<const double2 *>(p), a = __ldcg(q), b = __ldcg(q + 1);
+    return dvec4{a.x, a.y, b.x, b.y};
+}
 __device__ __forceinline__ double dot4(const double (&a)[4], const double (&b)[4])
 {
     return a[0] * b[0] + a[1] * b[1] + a[2] * b[2] + a[3] * b[3];
@@ -234,11 +247,32 @@ __device__ __forceinline__ void correct_sites(const F64Params &p, int cur, int f
         size_t s = (size_t)(2 + x) * sx + (size_t)y * p.n2 + z;
         for (int i = 0; i < len; ++i, s += sx) {
             dvec4 v, f;
-            arrest_fix_site(load4<double>(vn + s), load4<double>(vo + s), load4<double>(fo + s), (double)fix, p.dt, v, f);
+            arrest_fix_site(ldcg4(vn + s), ldcg4(vo + s), ldcg4(fo + s), (double)fix, p.dt, v, f);
             store4<double>(vn + s, v);
             store4<double>(fn + s, f);
         }
     }
+}
+
+__device__ __forceinline__ void st_release_s32(int *p, int v)
+{
+    asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ int ld_acquire_s32(const int *p)
+{
+    int v;
+    asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+// Polls until f() or the wait limit; whether f() came true.
+template <typename F> __device__ __forceinline__ bool wait_until(F f)
+{
+    if (f()) return true;
+    const unsigned long long t0 = global_ns();
+    do {
+        if (f()) return true;
+    } while (global_ns() - t0 < kWaitLimitNs);
+    return false;
 }
 
 template <bool EXT, int TZ>
@@ -253,230 +287,243 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_step_f64(const __grid_con
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // the previous launch is complete and visible from here on
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int cur = __ldcg(&p.ctrl->cur);
-    const int pred = p.mode == MODE_ARRESTED ? __ldcg(&p.ctrl->pred) : 0;
-    const long long steps0 = p.fuse_fix && tid == 0 ? ld_acquire_s64(&p.ctrl->steps) : 0;
-    const dvec4 *__restrict__ phi = cur ? p.phi[1] : p.phi[0];
-    const dvec4 *__restrict__ vin = cur ? p.vel[1] : p.vel[0];
-    dvec4 *__restrict__ phi_out = cur ? p.phi[0] : p.phi[1];
-    dvec4 *__restrict__ vel_out = cur ? p.vel[0] : p.vel[1];
-    const bool use_v = !pred;
-    const size_t sx = (size_t)p.n1 * p.n2;
-    // this warp's units, a contiguous range
-    const int wid = blockIdx.x * warps + warp, u0 = p.start[wid], u1 = p.start[wid + 1];
-    double acc[kSums64];
+    int cur = __ldcg(&p.ctrl->cur);
+    long long steps0 = tid == 0 ? ld_acquire_s64(&p.ctrl->steps) : 0;
+    for (int step = 1;; ++step, cur ^= 1) {
+        const int pred = p.mode == MODE_ARRESTED ? __ldcg(&p.ctrl->pred) : 0;
+        const dvec4 *phi = cur ? p.phi[1] : p.phi[0], *vin = cur ? p.vel[1] : p.vel[0];
+        dvec4 *phi_out = cur ? p.phi[0] : p.phi[1], *vel_out = cur ? p.vel[0] : p.vel[1];
+        const bool use_v = !pred;
+        const size_t sx = (size_t)p.n1 * p.n2;
+        // this warp's units, a contiguous range
+        const int wid = blockIdx.x * warps + warp, u0 = p.start[wid], u1 = p.start[wid + 1];
+        double acc[kSums64];
 #pragma unroll
-    for (int q = 0; q < kSums64; ++q) acc[q] = 0.0;
-    long long mx = 0;  // bits of max |F / 2B|^2
+        for (int q = 0; q < kSums64; ++q) acc[q] = 0.0;
+        long long mx = 0;  // bits of max |F / 2B|^2
 
-    for (int us = u0; us < u1;) {
-        const int col = us / p.nix, xs = 2 + (us - col * p.nix), xe = 2 + min(u1 - col * p.nix, p.nix);
-        us += xe - xs;
-        const Column c = column_at<TZ>(p, col);
-        const int y = c.y0 + ly, z = c.z0 + lz;
-        const bool valid = y <= p.n1 - 3 && z <= p.n2 - 3;
-        // this lane's copies of a haloed plane: byte offsets in the plane
-        // (sites outside the lattice are not read; only lanes that are not
-        // valid would use them)
-        int off[S::COPIES];
+        for (int us = u0; us < u1;) {
+            const int col = us / p.nix, xs = 2 + (us - col * p.nix), xe = 2 + min(u1 - col * p.nix, p.nix);
+            us += xe - xs;
+            const Column c = column_at<TZ>(p, col);
+            const int y = c.y0 + ly, z = c.z0 + lz;
+            const bool valid = y <= p.n1 - 3 && z <= p.n2 - 3;
+            // this lane's copies of a haloed plane: byte offsets in the plane
+            // (sites outside the lattice are not read; only lanes that are not
+            // valid would use them)
+            int off[S::COPIES];
 #pragma unroll
-        for (int j = 0; j < S::COPIES; ++j) {
-            const int i = lane + 32 * j, site = i >> 1, ry = site / S::RZ, rz = site - ry * S::RZ;
-            const int gy = c.y0 - 2 + ry, gz = c.z0 - 2 + rz;
-            off[j] = site < S::SITES && gy < p.n1 && gz < p.n2 ? (gy * p.n2 + gz) * 2 + (i & 1) : -1;
-        }
-        auto fetch = [&](int x) {
-            const double2 *src = reinterpret_cast<const double2 *>(phi + (size_t)x * sx);
-            const uint32_t dst = smem_u32(&ws.plane[x % kPlaneSlots][0]) + 16 * lane;
-#pragma unroll
-            for (int j = 0; j < S::COPIES; ++j)
-                if (off[j] >= 0)
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 512 * j),
-                                 "l"(__cvta_generic_to_global(src + off[j]))
-                                 : "memory");
-            asm volatile("cp.async.commit_group;" ::: "memory");
-        };
-        int next = xs - 2;  // the next plane to fetch
-        while (next < min(xs + 2, xe + 2)) fetch(next++);
-        dvec4 r[5] = {};  // phi at x - 2 .. x + 2 of the centre x = q - 2
-        const size_t col_site = (size_t)y * p.n2 + z;
-        for (int q = xs - 2; q < xe + 2; ++q) {
-            // plane q lands: the planes fetched after it may still be on their way
-            switch (next - 1 - q) {
-            case 0: asm volatile("cp.async.wait_group 0;" ::: "memory"); break;
-            case 1: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
-            case 2: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
-            default: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
+            for (int j = 0; j < S::COPIES; ++j) {
+                const int i = lane + 32 * j, site = i >> 1, ry = site / S::RZ, rz = site - ry * S::RZ;
+                const int gy = c.y0 - 2 + ry, gz = c.z0 - 2 + rz;
+                off[j] = site < S::SITES && gy < p.n1 && gz < p.n2 ? (gy * p.n2 + gz) * 2 + (i & 1) : -1;
             }
-            __syncwarp();
-            // the next plane's slot is free when its plane of four before has
-            // been a centre, or, at the start of a run, has arrived
-            if (next < xe + 2 && q >= (next - 4 < xs ? next - 3 : next - 1)) fetch(next++);
-            const int x = q - 2;
-            const bool centre = x >= xs;
-            dvec4 v = {0.0, 0.0, 0.0, 0.0};
-            if (centre && use_v && valid) v = load4<double>(vin + (size_t)x * sx + col_site);
-            {
-                // ---- plane q arrives: u_y (with its z-halo) and u_z
-                const dvec4 *P = &ws.plane[q % kPlaneSlots][0];
-                auto at = [&](int ry, int rz) { return lds(P + ry * S::RZ + rz); };
-                const dvec4 c4 = at(ly + 2, lz + 2);
-                r[0] = r[1], r[1] = r[2], r[2] = r[3], r[3] = r[4], r[4] = c4;
-                store4<double>(&ws.uy[q % 5][ly][lz + 2],
-                               first(at(ly, lz + 2), at(ly + 1, lz + 2), at(ly + 3, lz + 2), at(ly + 4, lz + 2)));
-                store4<double>(&ws.uz[q % 5][lane],
-                               first(at(ly + 2, lz), at(ly + 2, lz + 1), at(ly + 2, lz + 3), at(ly + 2, lz + 4)));
+            auto fetch = [&](int x) {
+                const double2 *src = reinterpret_cast<const double2 *>(phi + (size_t)x * sx);
+                const uint32_t dst = smem_u32(&ws.plane[x % kPlaneSlots][0]) + 16 * lane;
 #pragma unroll
-                for (int j = 0; j < S::HALO; ++j) {
-                    const int i = lane + 32 * j, hy = i >> 4, hc = (i >> 2) & 3, k = i & 3;
-                    const int hz = hc < 2 ? hc : TZ + hc;
-                    const double *b = reinterpret_cast<const double *>(P + hy * S::RZ + hz) + k;
-                    reinterpret_cast<double *>(&ws.uy[q % 5][hy][hz])[k] =
-                        first(b[0], b[4 * S::RZ], b[12 * S::RZ], b[16 * S::RZ]);
+                for (int j = 0; j < S::COPIES; ++j)
+                    if (off[j] >= 0)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 512 * j),
+                                     "l"(__cvta_generic_to_global(src + off[j]))
+                                     : "memory");
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            };
+            int next = xs - 2;  // the next plane to fetch
+            while (next < min(xs + 2, xe + 2)) fetch(next++);
+            dvec4 r[5] = {};  // phi at x - 2 .. x + 2 of the centre x = q - 2
+            const size_t col_site = (size_t)y * p.n2 + z;
+            for (int q = xs - 2; q < xe + 2; ++q) {
+                // plane q lands: the planes fetched after it may still be on their way
+                switch (next - 1 - q) {
+                case 0: asm volatile("cp.async.wait_group 0;" ::: "memory"); break;
+                case 1: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
+                case 2: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
+                default: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
+                }
+                __syncwarp();
+                // the next plane's slot is free when its plane of four before has
+                // been a centre, or, at the start of a run, has arrived
+                if (next < xe + 2 && q >= (next - 4 < xs ? next - 3 : next - 1)) fetch(next++);
+                const int x = q - 2;
+                const bool centre = x >= xs;
+                dvec4 v = {0.0, 0.0, 0.0, 0.0};
+                if (centre && use_v && valid) v = ldcg4(vin + (size_t)x * sx + col_site);
+                {
+                    // ---- plane q arrives: u_y (with its z-halo) and u_z
+                    const dvec4 *P = &ws.plane[q % kPlaneSlots][0];
+                    auto at = [&](int ry, int rz) { return lds(P + ry * S::RZ + rz); };
+                    const dvec4 c4 = at(ly + 2, lz + 2);
+                    r[0] = r[1], r[1] = r[2], r[2] = r[3], r[3] = r[4], r[4] = c4;
+                    store4<double>(&ws.uy[q % 5][ly][lz + 2],
+                                   first(at(ly, lz + 2), at(ly + 1, lz + 2), at(ly + 3, lz + 2), at(ly + 4, lz + 2)));
+                    store4<double>(&ws.uz[q % 5][lane],
+                                   first(at(ly + 2, lz), at(ly + 2, lz + 1), at(ly + 2, lz + 3), at(ly + 2, lz + 4)));
+#pragma unroll
+                    for (int j = 0; j < S::HALO; ++j) {
+                        const int i = lane + 32 * j, hy = i >> 4, hc = (i >> 2) & 3, k = i & 3;
+                        const int hz = hc < 2 ? hc : TZ + hc;
+                        const double *b = reinterpret_cast<const double *>(P + hy * S::RZ + hz) + k;
+                        reinterpret_cast<double *>(&ws.uy[q % 5][hy][hz])[k] =
+                            first(b[0], b[4 * S::RZ], b[12 * S::RZ], b[16 * S::RZ]);
+                    }
+                }
+                if (!centre) continue;  // (the same for the whole warp)
+                // ---- centre x: u_y's halo was written two planes ago
+                const dvec4 *P = &ws.plane[x % kPlaneSlots][0];
+                auto at = [&](int ry, int rz) { return lds(P + ry * S::RZ + rz); };
+                double ph[4], u[3][4], N[3][4], M[3][4], F[4], dens[5];
+                vec(ph, r[2]);
+                first(u[0], r[0], r[1], r[3], r[4]);
+                second(N[0], r[0], r[1], r[2], r[3], r[4]);
+                second(N[1], at(ly, lz + 2), at(ly + 1, lz + 2), r[2], at(ly + 3, lz + 2), at(ly + 4, lz + 2));
+                second(N[2], at(ly + 2, lz), at(ly + 2, lz + 1), r[2], at(ly + 2, lz + 3), at(ly + 2, lz + 4));
+                const int s0 = x % 5, m2 = (x + 3) % 5, m1 = (x + 4) % 5, p1 = (x + 1) % 5, p2 = (x + 2) % 5;
+                vec(u[1], lds(&ws.uy[s0][ly][lz + 2]));
+                vec(u[2], lds(&ws.uz[s0][lane]));
+                first(M[0], lds(&ws.uy[m2][ly][lz + 2]), lds(&ws.uy[m1][ly][lz + 2]), lds(&ws.uy[p1][ly][lz + 2]),
+                      lds(&ws.uy[p2][ly][lz + 2]));
+                first(M[1], lds(&ws.uz[m2][lane]), lds(&ws.uz[m1][lane]), lds(&ws.uz[p1][lane]), lds(&ws.uz[p2][lane]));
+                first(M[2], lds(&ws.uy[s0][ly][lz]), lds(&ws.uy[s0][ly][lz + 1]), lds(&ws.uy[s0][ly][lz + 3]),
+                      lds(&ws.uy[s0][ly][lz + 4]));
+                step_site<EXT>(p, ph, u, N, M, F, dens);
+                v = dvec4{::fma(p.dt2, F[0], v.x), ::fma(p.dt2, F[1], v.y), ::fma(p.dt2, F[2], v.z),
+                          ::fma(p.dt2, F[3], v.w)};
+                const double t[4] = {::fma(p.dt, v.x, ph[0]), ::fma(p.dt, v.y, ph[1]), ::fma(p.dt, v.z, ph[2]),
+                                     ::fma(p.dt, v.w, ph[3])};
+                const double rn = rsqrt(dot4(t, t));  // within an ulp of 1/sqrt, without its division
+                if (valid) {
+                    const size_t site = (size_t)x * sx + col_site;
+                    store4<double>(vel_out + site, v);
+                    store4<double>(phi_out + site, dvec4{t[0] * rn, t[1] * rn, t[2] * rn, t[3] * rn});
+                    const double f2 = dot4(F, F);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) acc[i] += dens[i];
+                    acc[4] += f2;
+                    mx = max(mx, __double_as_longlong(f2));  // (f2 >= 0: ordered as its bits)
+                    if constexpr (EXT) acc[6] += dens[4];
                 }
             }
-            if (!centre) continue;  // (the same for the whole warp)
-            // ---- centre x: u_y's halo was written two planes ago
-            const dvec4 *P = &ws.plane[x % kPlaneSlots][0];
-            auto at = [&](int ry, int rz) { return lds(P + ry * S::RZ + rz); };
-            double ph[4], u[3][4], N[3][4], M[3][4], F[4], dens[5];
-            vec(ph, r[2]);
-            first(u[0], r[0], r[1], r[3], r[4]);
-            second(N[0], r[0], r[1], r[2], r[3], r[4]);
-            second(N[1], at(ly, lz + 2), at(ly + 1, lz + 2), r[2], at(ly + 3, lz + 2), at(ly + 4, lz + 2));
-            second(N[2], at(ly + 2, lz), at(ly + 2, lz + 1), r[2], at(ly + 2, lz + 3), at(ly + 2, lz + 4));
-            const int s0 = x % 5, m2 = (x + 3) % 5, m1 = (x + 4) % 5, p1 = (x + 1) % 5, p2 = (x + 2) % 5;
-            vec(u[1], lds(&ws.uy[s0][ly][lz + 2]));
-            vec(u[2], lds(&ws.uz[s0][lane]));
-            first(M[0], lds(&ws.uy[m2][ly][lz + 2]), lds(&ws.uy[m1][ly][lz + 2]), lds(&ws.uy[p1][ly][lz + 2]),
-                  lds(&ws.uy[p2][ly][lz + 2]));
-            first(M[1], lds(&ws.uz[m2][lane]), lds(&ws.uz[m1][lane]), lds(&ws.uz[p1][lane]), lds(&ws.uz[p2][lane]));
-            first(M[2], lds(&ws.uy[s0][ly][lz]), lds(&ws.uy[s0][ly][lz + 1]), lds(&ws.uy[s0][ly][lz + 3]),
-                  lds(&ws.uy[s0][ly][lz + 4]));
-            step_site<EXT>(p, ph, u, N, M, F, dens);
-            v = dvec4{::fma(p.dt2, F[0], v.x), ::fma(p.dt2, F[1], v.y), ::fma(p.dt2, F[2], v.z),
-                      ::fma(p.dt2, F[3], v.w)};
-            const double t[4] = {::fma(p.dt, v.x, ph[0]), ::fma(p.dt, v.y, ph[1]), ::fma(p.dt, v.z, ph[2]),
-                                 ::fma(p.dt, v.w, ph[3])};
-            const double rn = rsqrt(dot4(t, t));  // within an ulp of 1/sqrt, without its division
-            if (valid) {
-                const size_t site = (size_t)x * sx + col_site;
-                store4<double>(vel_out + site, v);
-                store4<double>(phi_out + site, dvec4{t[0] * rn, t[1] * rn, t[2] * rn, t[3] * rn});
-                const double f2 = dot4(F, F);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) acc[i] += dens[i];
-                acc[4] += f2;
-                mx = max(mx, __double_as_longlong(f2));  // (f2 >= 0: ordered as its bits)
-                if constexpr (EXT) acc[6] += dens[4];
-            }
+            __syncwarp();  // the run's planes are done with before the next run's first arrives
         }
-        __syncwarp();  // the run's planes are done with before the next run's first arrives
-    }
 
-    // ---- sums: each warp's quantities over its lanes, then the CTA's warps
-    {
+        // ---- sums: each warp's quantities over its lanes, then the CTA's warps
+        {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        // three exchanges leave each lane one of the eight quantities
+            for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            // three exchanges leave each lane one of the eight quantities
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1) {
-            const bool up = lane & o;
+            for (int o = 4; o > 0; o >>= 1) {
+                const bool up = lane & o;
 #pragma unroll
-            for (int q = 0; q < o; ++q) {
-                const double keep = up ? acc[q + o] : acc[q], send = up ? acc[q] : acc[q + o];
-                acc[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                for (int q = 0; q < o; ++q) {
+                    const double keep = up ? acc[q + o] : acc[q], send = up ? acc[q] : acc[q + o];
+                    acc[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                }
             }
+            double v = acc[0];  // of quantity lane & 7
+            v += __shfl_xor_sync(0xffffffffu, v, 8);
+            v += __shfl_xor_sync(0xffffffffu, v, 16);
+            if (lane < kSums64) sm.red[warp][lane] = lane == 5 ? __longlong_as_double(mx) : v;
         }
-        double v = acc[0];  // of quantity lane & 7
-        v += __shfl_xor_sync(0xffffffffu, v, 8);
-        v += __shfl_xor_sync(0xffffffffu, v, 16);
-        if (lane < kSums64) sm.red[warp][lane] = lane == 5 ? __longlong_as_double(mx) : v;
-    }
-    __syncthreads();
-    if (tid < kSums64) {
-        double v = sm.red[0][tid];
-        for (int w = 1; w < warps; ++w) v = tid == 5 ? fmax(v, sm.red[w][tid]) : v + sm.red[w][tid];
-        p.parts[(size_t)blockIdx.x * kPartialDoubles + tid] = v;
-        __threadfence();
-    }
-    __syncthreads();
-    if (tid == 0) sm.last = atomicAdd(&p.ctrl->done, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (sm.last) {
-        // ---- the last CTA sums the records, 4 threads per warp and quantity;
-        // thread 0 fetches the control fields it needs meanwhile
-        __threadfence();
-        StepControl ctl;
-        if (tid == 0) ctl = load_control(p.ctrl);
-        const int q = tid & 7;
-        double v = 0.0;
-        for (int i0 = tid >> 3; i0 < (int)gridDim.x; i0 += 32 * warps) {
-            double t[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int i = i0 + 4 * warps * j;
-                t[j] = i < (int)gridDim.x ? __ldcg(p.parts + (size_t)i * kPartialDoubles + q) : 0.0;
-            }
-            if (q == 5) {
-#pragma unroll
-                for (int j = 0; j < 8; ++j) v = fmax(v, t[j]);
-            } else {
-                v += ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
-            }
-        }
-#pragma unroll
-        for (int o = 8; o <= 16; o <<= 1) {
-            const double t = __shfl_xor_sync(0xffffffffu, v, o);
-            v = q == 5 ? fmax(v, t) : v + t;
-        }
-        if (lane < kSums64) sm.red[warp][lane] = v;
         __syncthreads();
         if (tid < kSums64) {
-            double t = sm.red[0][tid];
-            for (int w = 1; w < warps; ++w) t = tid == 5 ? fmax(t, sm.red[w][tid]) : t + sm.red[w][tid];
-            sm.tot[tid] = t * p.scale[tid];
+            double v = sm.red[0][tid];
+            for (int w = 1; w < warps; ++w) v = tid == 5 ? fmax(v, sm.red[w][tid]) : v + sm.red[w][tid];
+            p.parts[(size_t)blockIdx.x * kPartialDoubles + tid] = v;
+            __threadfence();
         }
         __syncthreads();
-        if (tid == 0 || tid == 32) {
-            // thread 0 decides and publishes, thread 32 forms the report
-            const double *t = sm.tot;
-            const double nsites = (double)(p.n0 - 4) * (double)(p.n1 - 4) * (double)(p.n2 - 4);
-            const double tot[kPartialDoubles] = {t[0], t[1], t[2], t[3], t[4], t[5], nsites, t[6]};
-            if (p.slab_rec) {
-                // one x-slab of a larger lattice: the arrest decision needs
-                // every slab's sums, so this step only leaves its record
-                if (tid == 0) {
+        if (tid == 0) sm.last = atomicAdd(&p.ctrl->done, 1u) == gridDim.x - 1;
+        __syncthreads();
+        if (sm.last) {
+            // ---- the last CTA sums the records, 4 threads per warp and quantity;
+            // thread 0 fetches the control fields it needs meanwhile
+            __threadfence();
+            StepControl ctl;
+            if (tid == 0) ctl = load_control(p.ctrl);
+            const int q = tid & 7;
+            double v = 0.0;
+            for (int i0 = tid >> 3; i0 < (int)gridDim.x; i0 += 32 * warps) {
+                double t[8];
 #pragma unroll
-                    for (int i = 0; i < kPartialDoubles; ++i) p.slab_rec[i] = tot[i];
-                    p.ctrl->done = 0;
+                for (int j = 0; j < 8; ++j) {
+                    const int i = i0 + 4 * warps * j;
+                    t[j] = i < (int)gridDim.x ? __ldcg(p.parts + (size_t)i * kPartialDoubles + q) : 0.0;
                 }
-            } else if (tid == 0) {
-                decide_step(p.ctrl, ctl, tot, p.h3, p.mode, pred);
-            } else {
-                report_step(p.ctrl, tot, p.h3);
+                if (q == 5) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) v = fmax(v, t[j]);
+                } else {
+                    v += ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
+                }
+            }
+#pragma unroll
+            for (int o = 8; o <= 16; o <<= 1) {
+                const double t = __shfl_xor_sync(0xffffffffu, v, o);
+                v = q == 5 ? fmax(v, t) : v + t;
+            }
+            if (lane < kSums64) sm.red[warp][lane] = v;
+            __syncthreads();
+            if (tid < kSums64) {
+                double t = sm.red[0][tid];
+                for (int w = 1; w < warps; ++w) t = tid == 5 ? fmax(t, sm.red[w][tid]) : t + sm.red[w][tid];
+                sm.tot[tid] = t * p.scale[tid];
+            }
+            __syncthreads();
+            if (tid == 0 || tid == 32) {
+                // thread 0 decides and publishes, thread 32 forms the report
+                const double *t = sm.tot;
+                const double nsites = (double)(p.n0 - 4) * (double)(p.n1 - 4) * (double)(p.n2 - 4);
+                const double tot[kPartialDoubles] = {t[0], t[1], t[2], t[3], t[4], t[5], nsites, t[6]};
+                if (p.slab_rec) {
+                    // one x-slab of a larger lattice: the arrest decision needs
+                    // every slab's sums, so this step only leaves its record
+                    if (tid == 0) {
+#pragma unroll
+                        for (int i = 0; i < kPartialDoubles; ++i) p.slab_rec[i] = tot[i];
+                        p.ctrl->done = 0;
+                    }
+                } else if (tid == 0) {
+                    decide_step(p.ctrl, ctl, tot, p.h3, p.mode, pred);
+                } else {
+                    report_step(p.ctrl, tot, p.h3);
+                }
             }
         }
-    }
-    if (!p.fuse_fix) return;
-    // ---- every CTA (all resident: a cooperative launch) waits, bounded, for
-    // the decision and corrects its own sites when the prediction was wrong
-    if (tid == 0) {
-        long long st = ld_acquire_s64(&p.ctrl->steps);
-        if (st == steps0) {
-            const unsigned long long t0 = global_ns();
-            do {
-                st = ld_acquire_s64(&p.ctrl->steps);
-            } while (st == steps0 && global_ns() - t0 < kWaitLimitNs);
+        const bool more = step < p.steps;
+        if (!p.fuse_fix && !more) return;
+        // ---- every CTA (all resident: a cooperative launch) waits, bounded, for
+        // the decision and corrects its own sites when the prediction was wrong
+        if (tid == 0) {
+            sm.fix = wait_until([&] { return ld_acquire_s64(&p.ctrl->steps) != steps0; }) ? __ldcg(&p.ctrl->fix) : 2;
+            ++steps0;
         }
-        sm.fix = st == steps0 ? 2 : __ldcg(&p.ctrl->fix);
-    }
-    __syncthreads();
-    const int fix = sm.fix;
-    if (fix == 2) {
-        if (tid == 0) atomicExch(&p.ctrl->status, (int)DEV_TIMEOUT);
-    } else if (fix != 0) {
-        correct_sites<TZ>(p, cur, fix, u0, u1, ly, lz);
+        __syncthreads();
+        const int fix = sm.fix;
+        if (fix == 2) {
+            if (tid == 0) atomicExch(&p.ctrl->status, (int)DEV_TIMEOUT);
+            return;
+        }
+        if (fix != 0) correct_sites<TZ>(p, cur, fix, u0, u1, ly, lz);
+        if (!more) return;
+        if (fix != 0) {
+            // the next step reads its neighbours' corrected sites: the last CTA to
+            // arrive clears the correction, which the others wait for
+            __syncthreads();
+            if (tid == 0) {
+                __threadfence();
+                if (atomicAdd(&p.ctrl->done, 1u) == gridDim.x - 1) {
+                    p.ctrl->done = 0;
+                    st_release_s32(&p.ctrl->fix, 0);
+                } else if (!wait_until([&] { return ld_acquire_s32(&p.ctrl->fix) == 0; })) {
+                    sm.fix = 2;
+                    atomicExch(&p.ctrl->status, (int)DEV_TIMEOUT);
+                }
+            }
+            __syncthreads();
+            if (sm.fix == 2) return;
+        }
     }
 }
 
@@ -552,7 +599,7 @@ static int plan_warps(long long units, int nix, int sms, int *start)
     return warps;
 }
 
-template <bool EXT, int TZ> static cudaError_t launch_shape(F64Params &p, int sms, cudaStream_t s)
+template <bool EXT, int TZ> static cudaError_t launch_shape(F64Params &p, int steps, int sms, cudaStream_t s)
 {
     using S = ColumnShape<TZ>;
     p.nzt = (p.n2 - 4 + TZ - 1) / TZ;
@@ -568,7 +615,7 @@ template <bool EXT, int TZ> static cudaError_t launch_shape(F64Params &p, int sm
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = p.fuse_fix;
+    attr[0].val.cooperative = p.fuse_fix || p.steps > 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     // The next step's CTAs start as this one's leave only where one fits on an
     // SM: with 4 warps two fit, and a graph then packs some SMs with two of the
@@ -582,10 +629,15 @@ template <bool EXT, int TZ> static cudaError_t launch_shape(F64Params &p, int sm
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, k_step_f64<EXT, TZ>, p);
+    for (int left = steps; left > 0; left -= p.steps) {
+        p.steps = std::min(p.steps, left);
+        e = cudaLaunchKernelEx(&cfg, k_step_f64<EXT, TZ>, p);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
-cudaError_t launch_step_f64(const skyrme_lattice &lat, const FlowArgs &a, cudaStream_t s)
+cudaError_t launch_steps_f64(const skyrme_lattice &lat, const FlowArgs &a, int steps, cudaStream_t s)
 {
     F64Params p = {};
     for (int i = 0; i < 2; ++i) {
@@ -599,6 +651,10 @@ cudaError_t launch_step_f64(const skyrme_lattice &lat, const FlowArgs &a, cudaSt
     p.nix = p.n0 - 4;
     p.mode = a.mode;
     p.fuse_fix = a.mode == SKYRME_ARRESTED && !a.slab_rec;
+    // A launch runs as many steps as update kLaunchSites sites, about 3 ms: more
+    // save nothing, and other streams' kernels start between launches.
+    const double sites = (double)(p.n0 - 4) * (p.n1 - 4) * (p.n2 - 4);
+    p.steps = a.slab_rec ? 1 : (int)std::max(1.0, std::min((double)steps, kLaunchSites / sites));
     const double k1 = 1.0 / (12.0 * a.h), k2 = k1 * k1, B = 12.0 * k2 * k2;
     p.dt = a.dt;
     p.dt2 = 2.0 * a.dt * B;
@@ -621,8 +677,8 @@ cudaError_t launch_step_f64(const skyrme_lattice &lat, const FlowArgs &a, cudaSt
     const long long iy = p.n1 - 4, iz = p.n2 - 4;
     const long long pad16 = (iy + 1) / 2 * 2 * ((iz + 15) / 16 * 16), pad8 = (iy + 3) / 4 * 4 * ((iz + 7) / 8 * 8);
     if (101 * pad8 < 100 * pad16)
-        return ext ? launch_shape<true, 8>(p, sms, s) : launch_shape<false, 8>(p, sms, s);
-    return ext ? launch_shape<true, 16>(p, sms, s) : launch_shape<false, 16>(p, sms, s);
+        return ext ? launch_shape<true, 8>(p, steps, sms, s) : launch_shape<false, 8>(p, steps, sms, s);
+    return ext ? launch_shape<true, 16>(p, steps, sms, s) : launch_shape<false, 16>(p, steps, sms, s);
 }
 
 }  // namespace skyrme

@@ -659,7 +659,7 @@ cudaError_t launch_step(const skyrme_lattice &lat, const FlowArgs &a, cudaStream
     // modes do (48^3 95 -> 73 us a step).
     if (lat.precision == 64 && a.mode == MODE_GRADIENT)
         return launch_tile<double, 0>(lat, make_params<double>(a, a.step_parts), nullptr, nullptr, s);
-    if (lat.precision == 64) return launch_step_f64(lat, a, s);
+    if (lat.precision == 64) return launch_steps_f64(lat, a, 1, s);
     return launch_tile<float, 0>(lat, make_params<float>(a, a.step_parts), nullptr, nullptr, s);
 }
 

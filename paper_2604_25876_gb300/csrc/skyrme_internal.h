@@ -70,7 +70,7 @@ skyrme_status on_current_device(const void *const *ptrs, int n);
 cudaError_t launch_step(const skyrme_lattice &lat, const FlowArgs &a, cudaStream_t s);
 // The FP64 step (flow_f64.cu; not for the gradient flow); a whole lattice in
 // ARRESTED mode corrects its own mispredicted decisions inside it.
-cudaError_t launch_step_f64(const skyrme_lattice &lat, const FlowArgs &a, cudaStream_t s);
+cudaError_t launch_steps_f64(const skyrme_lattice &lat, const FlowArgs &a, int steps, cudaStream_t s);
 cudaError_t launch_fixup(const skyrme_lattice &lat, const FlowArgs &a, cudaStream_t s);
 cudaError_t launch_energy(const skyrme_lattice &lat, const FlowArgs &a, cudaStream_t s);
 cudaError_t launch_forces(const skyrme_lattice &lat, const FlowArgs &a, void *force, void *dens,

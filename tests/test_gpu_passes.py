@@ -222,6 +222,23 @@ def test_fp64_steps_match_oracle_at_the_edges_of_the_work_split(n, mode, model):
     assert rep["steps"] == steps and rep["status"] == 0
 
 
+# several FP64 steps in a launch: fewer and more units than CTAs, both column
+# shapes; time steps that arrest often, so that decisions are mispredicted
+@pytest.mark.parametrize("n", [(7, 8, 21), (20, 22, 24), (24, 48, 48), (70, 66, 68)])
+@pytest.mark.parametrize("mode,dt", [(sk.ARRESTED, 0.03), (sk.NEWTON, 0.004)])
+def test_fp64_steps_of_one_call_equal_single_steps(n, mode, dt):
+    h, steps = 0.25, 33
+    lat, one, phi = on_gpu(field(n, h, 2), h, 64)
+    _, many, _ = on_gpu(phi, h, 64)
+    for _ in range(steps):
+        a = sk.flow_step(lat, dt, 1, mode, one)
+    b = sk.flow_step(lat, dt, steps, mode, many)
+    assert a == b and b["steps"] == steps and b["status"] == 0
+    assert torch.equal(one.phi, many.phi) and torch.equal(one.vel, many.vel)
+    if mode == sk.ARRESTED and min(n) > 8:
+        assert b["fixups"] > 0
+
+
 @pytest.mark.parametrize("n", SIZES + [(6, 40, 52)])
 @pytest.mark.parametrize("prec", [64, 32])
 def test_load_field_gives_the_same_state_from_every_source(n, prec):
