@@ -53,8 +53,8 @@ FLOPS_PER_SITE_POT = 638  # potentials only (the standard count + their 17-opera
 # FP64 operations (FMA = 2) the diagnostic kernels execute, from ncu op
 # counts (dadd + dmul + 2 dfma) on the 128^3 field; each formula is evaluated
 # once per site and pass, so these are their arithmetic:
-OBS_FP64_FLOPS_PER_SITE = 1032          # Section 5 observables: 124 + 908 per interior site
-RENDER_VOLUME_FP64_FLOPS_PER_SITE = 183  # volume record + normalisation, per lattice site
+OBS_FP64_FLOPS_PER_SITE = 585           # Section 5 observables: 107 + 478 per interior site
+RENDER_VOLUME_FP64_FLOPS_PER_SITE = 149  # volume record + normalisation, per lattice site
 GRAPH_CHUNK = 250         # iterations per captured CUDA graph
 
 
@@ -121,18 +121,21 @@ def flops_per_site(wl):
 
 def step_kernel_key(wl, prec):
     """Name of the step kernel a workload runs on (the traffic record key):
-    the FP32 streaming kernel for the standard model and the potentials, the
-    tile kernels for FP64 and for the sextic term."""
+    the FP32 streaming kernel or the FP64 one (two key prefixes: the standard
+    model, and the extended models' instantiation)."""
     if prec == 32 and wl.streaming:
         return f"step_f32_{wl.name}"
     return f"step_tile_f{prec}_{wl.name}" if wl.extended else f"step_f64_{wl.name}"
 
 
-def launches_per_step(wl, prec):
-    """Kernel launches of one ARRESTED iteration: the FP32 streaming step
-    corrects its own arrest mispredictions; the tile kernels (FP64, the
-    sextic term) are followed by a fix-up check launch."""
-    return 1 if (prec == 32 and wl.streaming) else 2
+def step_launches(wl, prec, steps):
+    """Kernel launches of a graph of ``steps`` ARRESTED iterations: one each for
+    the FP32 streaming step, and for the FP64 step one for as many iterations as
+    update 2^22 sites (both correct their own mispredictions); with a fix-up
+    check each for the FP32 tile step."""
+    if prec == 64:
+        return math.ceil(steps / max(1, min(steps, (1 << 22) // wl.interior_sites)))
+    return steps if wl.streaming else 2 * steps
 
 
 def l2_note(wl):
@@ -225,11 +228,11 @@ def source_code_only(text: str) -> str:
 
 def kernel_fingerprint(kernel_key: str):
     """Hash of the code of a step kernel's sources: the FP32 streaming
-    kernel (keys step_f32_*) or the tile kernels (every other key), with
+    kernel (keys step_f32_*) or the FP64 step (every other key), with
     their shared header; comments and layout do not count."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2604_25876_gb300", "csrc")
-    src = "flow_f32.cu" if kernel_key.startswith("step_f32_") else "flow_generic.cu"
+    src = "flow_f32.cu" if kernel_key.startswith("step_f32_") else "flow_f64.cu"
     for name in (src, "skyrme_device.cuh"):
         with open(os.path.join(csrc, name), encoding="utf-8") as f:
             h.update(source_code_only(f.read()).encode())
@@ -369,7 +372,7 @@ def run_ours(args, ws, rank, local):
            "scaling": "weak", "vs_baseline": None, "dtype": "f32" if prec == 32 else "f64",
            "data": "synthetic",
            "config": workload_config(wl), "roofline": roofline,
-           "gpu_launches": launches_per_step(wl, prec) * K, "graph_chunk": chunk, "clocks": clk,
+           "gpu_launches": sum(step_launches(wl, prec, g.nsteps) for g in plan), "graph_chunk": chunk, "clocks": clk,
            "repeats": spread(repeats, f"{len(repeats)} more passes of the same {K} graph-replayed "
                                       "iterations, each continuing the flow"),
            "flow": {"steps_done": rep["steps"], "arrests": rep["arrests"],

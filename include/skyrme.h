@@ -62,8 +62,8 @@ typedef enum { SKYRME_NEWTON = 0, SKYRME_ARRESTED = 1, SKYRME_GRADIENT = 2 } sky
  * non-zero is an "extended" lattice: the Section 5 observables reject it with
  * SKYRME_EUNSUPPORTED, and so does the batched flow when c6 != 0 (batches
  * take the standard model and the potentials).  An FP32 flow runs on the
- * streaming FP32 kernel with any of the terms; an FP64 flow runs on the tile
- * kernels. */
+ * streaming FP32 kernel with any of the terms; an FP64 flow on the FP64 step
+ * kernel. */
 typedef struct {
     int n[3];       /* sites per axis (x slowest, z fastest); each >= 5 */
     double h;       /* lattice spacing, > 0, equal on every axis */
