@@ -327,11 +327,13 @@ __global__ void __launch_bounds__(256) k_seed_product(vec4_t<T> *phi0, vec4_t<T>
 // U_1 ... U_k and the conjugate of U_k ... U_1 are the two halves of the
 // packed FP32 instructions: the second is the product of the conjugates.
 //
-// Bound by the FP32 pipe (about 85% busy; 400 warp instructions per 32 sites and
-// constituent, three quarters of them FP32, most of those packed).  FP64 and
-// double-float, symmetrised: 256^3 with 8 constituents 17.6 and 2.35 ms, with one
-// 2.07 and 0.53 ms (268 MB written four times: 0.16 ms); 151^3 with 4 constituents
-// 1.84 and 0.33 ms; 128^3 with 64 constituents 17.5 and 3.3 ms.
+// Bound by issue and the FP32 pipe (59% and 62% busy with 16 warps per SM; 336
+// warp instructions per 32 sites and constituent, 240 of them FP32, most of those
+// packed; 20 and 24 warps with fewer registers were 3% slower).  FP64 and
+// double-float, symmetrised: 256^3 with 8 constituents 17.6 and 2.02 ms (2.35 with
+// products and their rounding errors formed before they are summed), with one
+// 2.07 and 0.51 ms (268 MB written four times: 0.16 ms); 151^3 with 4 constituents
+// 1.84 and 0.30 ms; 128^3 with 64 constituents 17.5 and 2.8 ms.
 constexpr int kPairOctaves = 22, kPairPerOctave = 256;  // q / scale^2 from 2^-12 to 2^10
 constexpr int kPairIntervals = kPairOctaves * kPairPerOctave;
 constexpr int kPairBase = (127 - 12) * kPairPerOctave;
@@ -339,7 +341,7 @@ constexpr int kPairVecs = 5;  // float4 per interval: (C, S) pairs hi, lo of deg
 constexpr size_t kPairTableBytes = (size_t)kPairIntervals * kPairVecs * sizeof(float4);
 // The bounds err[] below: the scalar component's error against 1, the others'
 // against the sum of the constituents' pion sizes.  Over lattice spacings of 0.02
-// to 2 scales and 1 to 64 constituents the largest error met was 0.15 of them.
+// to 2 scales and 1 to 64 constituents the largest error met was 0.22 of them.
 constexpr float kPairEps = 0x1p-40f;
 
 __global__ void k_pair_table(float4 *table)
@@ -352,8 +354,10 @@ __global__ void k_pair_table(float4 *table)
     float4 *t = table + i * kPairVecs;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const float c = (float)C[k], v = (float)S[k];
-        t[k] = make_float4(c, v, (float)(C[k] - (double)c), (float)(S[k] - (double)v));
+        // C itself passes through 0: its hi part is kept as 3 + hi, exactly
+        const double off = k == 0 ? 3.0 : 0.0;
+        const float c = (float)(C[k] + off), v = (float)S[k];
+        t[k] = make_float4(c, v, (float)(C[k] - ((double)c - off)), (float)(S[k] - (double)v));
     }
     t[3] = make_float4((float)C[3], (float)S[3], (float)C[4], (float)S[4]);
     t[4] = make_float4((float)C[5], (float)S[5], (float)C[6], (float)S[6]);
@@ -361,68 +365,53 @@ __global__ void k_pair_table(float4 *table)
 
 // -x off the FP32 pipe
 __device__ __forceinline__ float neg(float x) { return __int_as_float(__float_as_int(x) ^ (int)0x80000000); }
-// s + e = a + b exactly
-__device__ __forceinline__ void two_sum(float2 a, float2 b, float2 &s, float2 &e)
+// (ch + cl) + (xh + xl)(d + dl), two quantities.  |ch| is above |xh d|, so that
+// ch - (the rounded sum) is exact and the rounding error one more FMA.
+__device__ __forceinline__ void horner(float2 ch, float2 cl, float2 &xh, float2 &xl, float2 d, float2 dl)
 {
-    const float2 m1 = bc(-1.f);
-    s = __fadd2_rn(a, b);
-    const float2 bb = __ffma2_rn(a, m1, s);                                               // s - a
-    e = __fadd2_rn(__ffma2_rn(__ffma2_rn(bb, m1, s), m1, a), __ffma2_rn(bb, m1, b));
-}
-// (ch + cl) + (xh + xl)(d + dl), two quantities; nd = -d
-__device__ __forceinline__ void horner(float2 ch, float2 cl, float2 &xh, float2 &xl, float2 d, float2 nd, float2 dl)
-{
-    const float2 n = __fmul2_rn(xh, nd);
-    float2 e = __ffma2_rn(xh, d, n);
+    const float2 s = __ffma2_rn(xh, d, ch);
+    float2 e = __ffma2_rn(xh, d, __ffma2_rn(s, bc(-1.f), ch));
     e = __ffma2_rn(xl, d, e);
     e = __ffma2_rn(xh, dl, e);
-    two_sum(ch, __fmul2_rn(xh, d), xh, xl);
-    xl = __fadd2_rn(xl, __fadd2_rn(cl, e));
+    xl = __fadd2_rn(cl, e);
+    xh = s;
 }
-// sum_j x_j y_j of pairs of double-floats, n = -y.  The products are added to
-// `shift`, 3 times a power of two above twice their partial sums: each addition
-// then rounds at the same place, and what it drops is exact in two operations.
+// sum_j x_j y_j of pairs of double-floats.  The products are added to `shift`,
+// above twice their partial sums: what a sum kept of a product is then exact in
+// one subtraction, and what it dropped one more FMA.
 struct Pairs4 {
     float2 h[4], l[4];
 };
 __device__ __forceinline__ void dot_pairs(const float2 (&xh)[4], const float2 (&xl)[4], const float2 (&y)[4],
-                                          const float2 (&ny)[4], const float2 (&nyl)[4], float2 shift, float2 &h,
-                                          float2 &l)
+                                          const float2 (&yl)[4], float2 shift, float2 &h, float2 &l)
 {
-    float2 p[4], n;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) p[j] = __fmul2_rn(xh[j], y[j]);
-    n = __ffma2_rn(xh[0], ny[0], p[0]);  // minus the product's rounding error
-#pragma unroll
-    for (int j = 1; j < 4; ++j) n = __fadd2_rn(n, __ffma2_rn(xh[j], ny[j], p[j]));
-#pragma unroll
-    for (int j = 0; j < 4; ++j) n = __ffma2_rn(xl[j], ny[j], __ffma2_rn(xh[j], nyl[j], n));
     const float2 m1 = bc(-1.f);
-    float2 s = shift;
+    float2 s = shift, n;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        const float2 t = __fadd2_rn(s, p[j]);
-        const float2 r = __ffma2_rn(s, m1, t);  // p_j as rounded
-        n = __fadd2_rn(n, __ffma2_rn(p[j], m1, r));
+        const float2 t = __ffma2_rn(xh[j], y[j], s);
+        const float2 e = __ffma2_rn(xh[j], y[j], __ffma2_rn(t, m1, s));
+        n = j == 0 ? e : __fadd2_rn(n, e);
         s = t;
     }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) n = __ffma2_rn(xl[j], y[j], __ffma2_rn(xh[j], yl[j], n));
     s = __ffma2_rn(shift, m1, s);
-    h = __ffma2_rn(n, m1, s);
-    l = __ffma2_rn(n, m1, __ffma2_rn(h, m1, s));
+    h = __fadd2_rn(s, n);
+    l = __ffma2_rn(__ffma2_rn(s, m1, h), m1, n);
 }
 // x y of two quantities' quaternions, y given with its negative
 __device__ __forceinline__ void mul_pairs(Pairs4 &x, const Pairs4 &y, const Pairs4 &n, float2 shift0, float2 shift)
 {
     Pairs4 r;
-    const auto row = [&](int i, float2 y0, float2 y1, float2 y2, float2 y3, float2 n0, float2 n1, float2 n2, float2 n3,
-                         float2 l0, float2 l1, float2 l2, float2 l3) {
-        const float2 yy[4] = {y0, y1, y2, y3}, nn[4] = {n0, n1, n2, n3}, nl[4] = {l0, l1, l2, l3};
-        dot_pairs(x.h, x.l, yy, nn, nl, i == 0 ? shift0 : shift, r.h[i], r.l[i]);
+    const auto row = [&](int i, float2 y0, float2 y1, float2 y2, float2 y3, float2 l0, float2 l1, float2 l2, float2 l3) {
+        const float2 yy[4] = {y0, y1, y2, y3}, ll[4] = {l0, l1, l2, l3};
+        dot_pairs(x.h, x.l, yy, ll, i == 0 ? shift0 : shift, r.h[i], r.l[i]);
     };
-    row(0, y.h[0], n.h[1], n.h[2], n.h[3], n.h[0], y.h[1], y.h[2], y.h[3], n.l[0], y.l[1], y.l[2], y.l[3]);
-    row(1, y.h[1], y.h[0], n.h[3], y.h[2], n.h[1], n.h[0], y.h[3], n.h[2], n.l[1], n.l[0], y.l[3], n.l[2]);
-    row(2, y.h[2], y.h[3], y.h[0], n.h[1], n.h[2], n.h[3], n.h[0], y.h[1], n.l[2], n.l[3], n.l[0], y.l[1]);
-    row(3, y.h[3], n.h[2], y.h[1], y.h[0], n.h[3], y.h[2], n.h[1], n.h[0], n.l[3], y.l[2], n.l[1], n.l[0]);
+    row(0, y.h[0], n.h[1], n.h[2], n.h[3], y.l[0], n.l[1], n.l[2], n.l[3]);
+    row(1, y.h[1], y.h[0], n.h[3], y.h[2], y.l[1], y.l[0], n.l[3], y.l[2]);
+    row(2, y.h[2], y.h[3], y.h[0], n.h[1], y.l[2], y.l[3], y.l[0], n.l[1]);
+    row(3, y.h[3], n.h[2], y.h[1], y.h[0], y.l[3], n.l[2], y.l[1], y.l[0]);
     x = r;
 }
 
@@ -463,18 +452,18 @@ __device__ __forceinline__ bool product_pairs(const float4 *ob, int K, const flo
         const float4 t0 = __ldg(t), t1 = __ldg(t + 1), t2 = __ldg(t + 2), t3 = __ldg(t + 3), t4 = __ldg(t + 4);
         // q from the interval's centre (the subtraction is exact)
         const DF dq = quick_two_sum(__fsub_rn(q.hi, __int_as_float((bits & ~0x7fff) | 0x4000)), q.lo);
-        const float2 d = bc(dq.hi), nd = bc(-dq.hi), dl = bc(dq.lo);
+        const float2 d = bc(dq.hi), dl = bc(dq.lo);
         float2 xh = __ffma2_rn(make_float2(t4.z, t4.w), d, make_float2(t4.x, t4.y));
         xh = __ffma2_rn(xh, d, make_float2(t3.z, t3.w));
         xh = __ffma2_rn(xh, d, make_float2(t3.x, t3.y));
         float2 xl = __ffma2_rn(xh, d, make_float2(t2.z, t2.w));
         xh = make_float2(t2.x, t2.y);
-        horner(make_float2(t1.x, t1.y), make_float2(t1.z, t1.w), xh, xl, d, nd, dl);
-        horner(make_float2(t0.x, t0.y), make_float2(t0.z, t0.w), xh, xl, d, nd, dl);
+        horner(make_float2(t1.x, t1.y), make_float2(t1.z, t1.w), xh, xl, d, dl);
+        horner(make_float2(t0.x, t0.y), make_float2(t0.z, t0.w), xh, xl, d, dl);
+        xh.x -= 3.f;
         // U_k and its conjugate
         Pairs4 y, n;
         y.h[0] = bc(xh.x), y.l[0] = bc(xl.x);
-        n.h[0] = bc(neg(xh.x)), n.l[0] = bc(neg(xl.x));
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             const float u = __fmul_rn(xh.y, ph[i]);
@@ -488,7 +477,7 @@ __device__ __forceinline__ bool product_pairs(const float4 *ob, int K, const flo
             x = y;
         } else {
             // the vector components' partial sums stay below 2 P, the scalar's below 1
-            const float big = __int_as_float(((__float_as_int(P) & 0x7f800000) + (3 << 23)) | 0x400000);
+            const float big = __int_as_float(((__float_as_int(P) & 0x7f800000) + (2 << 23)) | 0x400000);
             mul_pairs(x, y, n, bc(3.f), bc(big));
         }
     }
@@ -843,7 +832,7 @@ static cudaError_t seed_impl(const skyrme_lattice &lat, const skyrme_seed &sd, c
             c.norm = r[0];
         }
         // The double-float kernel takes 60 us at least (its table, the FP64
-        // remainder): 64^3 with one constituent 64 us against 79, 32^3 with eight
+        // remainder): 64^3 with one constituent 66 us against 79, 32^3 with eight
         // 91 against 93, 50^3 with one 60 against 60.
         const double work = (double)total * sd.B;
         if (sizeof(T) == 4 && work >= 2.5e5 && pairs_apply(lat, pa)) return launch_product_f32(lat, pa, sd.symmetrise, a, s);
