@@ -264,10 +264,12 @@ skyrme_status skyrme_init_field(const skyrme_lattice *lat, const skyrme_seed *se
     CKDEV(state_on_device(st));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     FlowArgs a = make_args(*lat, *st, 0.0, MODE_ARRESTED);
-    CK(launch_reset_ctrl(a.ctrl, s), "reset control block");
+    // the noise seed counts its blocks in the control block, which the load
+    // then resets; the product seed writes the whole state itself
+    const bool product = seed->kind == SKYRME_SEED_PRODUCT;
+    if (product || seed->kind == SKYRME_SEED_NOISE) CK(launch_reset_ctrl(a.ctrl, s), "reset control block");
     CK(launch_seed(*lat, *seed, a, s), "seed kernels");
-    // (the product seed writes the whole state itself)
-    if (seed->kind != SKYRME_SEED_PRODUCT) CK(launch_load_finish(*lat, a, s), "finish field");
+    if (!product) CK(launch_load_finish(*lat, a, s), "finish field");
     return SKYRME_OK;
 }
 
@@ -278,7 +280,6 @@ skyrme_status skyrme_load_field(const skyrme_lattice *lat, skyrme_state *st, voi
     CKDEV(state_on_device(st));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     FlowArgs a = make_args(*lat, *st, 0.0, MODE_ARRESTED);
-    CK(launch_reset_ctrl(a.ctrl, s), "reset control block");
     CK(launch_load_finish(*lat, a, s), "finish field");
     return SKYRME_OK;
 }
@@ -299,7 +300,6 @@ skyrme_status skyrme_load_field_from(const skyrme_lattice *lat, skyrme_state *st
     CKDEV(on_current_device(&src, 1));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     FlowArgs a = make_args(*lat, *st, 0.0, MODE_ARRESTED);
-    CK(launch_reset_ctrl(a.ctrl, s), "reset control block");
     CK(launch_load_finish(*lat, a, s, src), "load field");
     return SKYRME_OK;
 }
@@ -430,7 +430,6 @@ skyrme_status skyrme_flow_host(const skyrme_lattice *lat, double dt, int nsteps,
     }
     if (direct) {
         FlowArgs l = make_args(*lat, *st, 0.0, MODE_ARRESTED);
-        CK(launch_reset_ctrl(l.ctrl, s), "reset control block");
         CK(launch_load_finish(*lat, l, s, direct), "load field from host");
     } else {
         CK(cudaMemcpyAsync(st->phi[0], field_in, bytes, cudaMemcpyHostToDevice, s), "upload field");

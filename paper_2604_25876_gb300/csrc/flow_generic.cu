@@ -449,8 +449,29 @@ template <typename T> __global__ void __launch_bounds__(512, 2) k_fixup(FlowPara
     }
 }
 
+// The control block of a state whose field has just been set.
+__device__ void reset_ctrl(Ctrl *c)
+{
+    c->E_prev = __longlong_as_double(0x7ff0000000000000LL);  // +inf
+    for (int i = 0; i < 8; ++i) c->last[i] = 0.0, c->energy[i] = 0.0;
+    c->steps = 0;
+    c->arrests = 0;
+    c->fixups = 0;
+    c->cur = 0;
+    c->pred = 0;
+    c->fix = 0;
+    c->status = 0;
+    c->done = 0;
+    c->edone = 0;
+    c->hist = 0;
+    for (int i = 0; i < 16; ++i) c->pht[i] = 1;  // weakly "no arrest"
+    c->until_start = 0;
+    c->e6_last = 0.0;
+    c->e6_energy = 0.0;
+}
+
 // The state of a field just loaded: phi[1] <- phi[0], the outer layers of both
-// the vacuum, velocities 0.  With a source (a caller's field on the device, or
+// the vacuum, velocities 0, the control block as new.  With a source (a caller's field on the device, or
 // in pinned host memory and then read over the host link) phi[0] <- src too;
 // without one the interior of phi[0] is not written again.
 // Bound by DRAM: one buffer read and three (with a source four) written.
@@ -461,6 +482,7 @@ template <typename T, bool SRC>
 __global__ void __launch_bounds__(256) k_load_field(FlowParams<T> p, const vec4_t<T> *__restrict__ src)
 {
     constexpr int kPer = 4;  // sites per thread and pass
+    if (blockIdx.x == 0 && threadIdx.x == 0) reset_ctrl(p.ctrl);
     const vec4_t<T> vac = make4<T>(T(1), T(0), T(0), T(0)), zero = make4<T>(T(0), T(0), T(0), T(0));
     const unsigned plane = (unsigned)p.n1 * p.n2, blocks = (plane + 256 * kPer - 1) / (256 * kPer);
     const unsigned items = blocks * p.n0;
@@ -493,24 +515,7 @@ __global__ void __launch_bounds__(256) k_load_field(FlowParams<T> p, const vec4_
 
 __global__ void k_reset_ctrl(Ctrl *c)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        c->E_prev = __longlong_as_double(0x7ff0000000000000LL);  // +inf
-        for (int i = 0; i < 8; ++i) c->last[i] = 0.0, c->energy[i] = 0.0;
-        c->steps = 0;
-        c->arrests = 0;
-        c->fixups = 0;
-        c->cur = 0;
-        c->pred = 0;
-        c->fix = 0;
-        c->status = 0;
-        c->done = 0;
-        c->edone = 0;
-        c->hist = 0;
-        for (int i = 0; i < 16; ++i) c->pht[i] = 1;  // weakly "no arrest"
-        c->until_start = 0;
-        c->e6_last = 0.0;
-        c->e6_energy = 0.0;
-    }
+    if (threadIdx.x == 0 && blockIdx.x == 0) reset_ctrl(c);
 }
 
 // Run-to-tolerance graphs: a WHILE node repeats a body of `chunk` iterations.
