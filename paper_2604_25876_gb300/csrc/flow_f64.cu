@@ -512,8 +512,12 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_step_f64(const __grid_con
             // arrive clears the correction, which the others wait for
             __syncthreads();
             if (tid == 0) {
+                // released before the arrival and acquired after it: the last CTA's
+                // release below then covers every CTA's corrected sites
                 __threadfence();
-                if (atomicAdd(&p.ctrl->done, 1u) == gridDim.x - 1) {
+                const bool last = atomicAdd(&p.ctrl->done, 1u) == gridDim.x - 1;
+                __threadfence();
+                if (last) {
                     p.ctrl->done = 0;
                     st_release_s32(&p.ctrl->fix, 0);
                 } else if (!wait_until([&] { return ld_acquire_s32(&p.ctrl->fix) == 0; })) {

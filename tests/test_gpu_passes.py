@@ -239,6 +239,31 @@ def test_fp64_steps_of_one_call_equal_single_steps(n, mode, dt):
         assert b["fixups"] > 0
 
 
+# the corrections of several steps in one launch, by every entry point that
+# runs them, for both instantiations of the step and both column shapes
+@pytest.mark.parametrize("n", [(20, 22, 24), (24, 48, 48)])
+@pytest.mark.parametrize("model,dt", [({}, 0.03), ({"m_y": 0.5, "m_z": 0.3, "m_w": 1.0, "c6": 0.02}, 0.02)])
+@pytest.mark.parametrize("entry", ["call", "graph", "until"])
+def test_fp64_corrections_in_a_launch_equal_single_steps(n, model, dt, entry):
+    h, steps = 0.25, 60
+    lat, one, phi = on_gpu(field(n, h, 2), h, 64, **model)
+    _, many, _ = on_gpu(phi, h, 64, **model)
+    for _ in range(steps):
+        a = sk.flow_step(lat, dt, 1, sk.ARRESTED, one)
+    if entry == "call":
+        b = sk.flow_step(lat, dt, steps, sk.ARRESTED, many)
+    elif entry == "graph":
+        g = sk.FlowGraph(lat, many, dt, steps, sk.ARRESTED)
+        g.launch()
+        b = many.report()
+        g.close()
+    else:
+        b = sk.flow_until(lat, dt, sk.ARRESTED, many, 0.0, steps, chunk=20)
+    assert a == b and b["steps"] == steps and b["status"] == 0
+    assert b["fixups"] > 1
+    assert torch.equal(one.phi, many.phi) and torch.equal(one.vel, many.vel)
+
+
 @pytest.mark.parametrize("n", SIZES + [(6, 40, 52)])
 @pytest.mark.parametrize("prec", [64, 32])
 def test_load_field_gives_the_same_state_from_every_source(n, prec):
