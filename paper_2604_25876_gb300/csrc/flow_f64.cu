@@ -32,9 +32,12 @@
 //    when sites were corrected.  One step per launch and now, us per step in a
 //    graph and on a stream: 24 x 26 x 28 26.9 and 29.2 -> 25.7 and 26.0, 48^3
 //    73.7 and 76.3 -> 72.5 and 73.0, 90 x 75 x 83 326 and 329 -> 325 and 325.
-//  * Consecutive launches are programmatic dependents (with 8 and 6 warps per
-//    CTA): a launch's CTAs start as the last one's leave, and wait for it before
-//    they read anything it wrote.
+//  * Launches whose CTAs wait for one another (for the decision, or for the next
+//    step) are cooperative: the CTAs of one are resident together, whatever other
+//    streams run.  Consecutive launches are not programmatic dependents, whose
+//    CTAs start one by one as the last launch's leave: two flows on two streams
+//    could then each hold some SMs and wait for CTAs that the other leaves no
+//    room for.
 //  * Measured (us per iteration, tile kernel and fix-up launch before -> now):
 //    48^3 103.6 -> 73, 64^3 187 -> 153, 128^3 1392 -> 1166 (1.63 G
 //    site-updates/s, 334 instructions per site at the measured FP64 FMA rate),
@@ -284,9 +287,6 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_step_f64(const __grid_con
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, warps = blockDim.x >> 5;
     WarpSmem<TZ> &ws = reinterpret_cast<WarpSmem<TZ> *>(smem_raw + sizeof(StepSmem64))[warp];
     const int ly = lane / TZ, lz = lane % TZ;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // the previous launch is complete and visible from here on
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     int cur = __ldcg(&p.ctrl->cur);
     long long steps0 = tid == 0 ? ld_acquire_s64(&p.ctrl->steps) : 0;
     for (int step = 1;; ++step, cur ^= 1) {
@@ -617,22 +617,16 @@ template <bool EXT, int TZ> static cudaError_t launch_shape(F64Params &p, int st
     while (used > 1 && p.start[used - 1] == p.units) --used;
     cudaError_t e = cudaFuncSetAttribute(k_step_f64<EXT, TZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
     if (e != cudaSuccess) return e;
-    cudaLaunchAttribute attr[2];
+    cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = p.fuse_fix || p.steps > 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    // The next step's CTAs start as this one's leave only where one fits on an
-    // SM: with 4 warps two fit, and a graph then packs some SMs with two of the
-    // next step's (48^3: 127 us a step instead of 74).
-    attr[1].val.programmaticStreamSerializationAllowed =
-        !p.slab_rec && 2 * (sizeof(StepSmem64) + warps * sizeof(WarpSmem<TZ>)) > 228 * 1024;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((used + warps - 1) / warps));
     cfg.blockDim = dim3(32 * warps);
     cfg.dynamicSmemBytes = sizeof(StepSmem64) + warps * sizeof(WarpSmem<TZ>);
     cfg.stream = s;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = 1;
     for (int left = steps; left > 0; left -= p.steps) {
         p.steps = std::min(p.steps, left);
         e = cudaLaunchKernelEx(&cfg, k_step_f64<EXT, TZ>, p);

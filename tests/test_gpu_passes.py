@@ -264,6 +264,32 @@ def test_fp64_corrections_in_a_launch_equal_single_steps(n, model, dt, entry):
     assert torch.equal(one.phi, many.phi) and torch.equal(one.vel, many.vel)
 
 
+# launches that wait inside (for the arrest decision, for the next step) on two
+# streams at a time: one or two CTAs to an SM, some SMs idle, different lattices
+@pytest.mark.parametrize("na,nb", [((48, 48, 48), (48, 48, 48)), ((20, 22, 24), (70, 66, 68)),
+                                   ((70, 66, 68), (66, 70, 64))])
+@pytest.mark.parametrize("mode,dt", [(sk.ARRESTED, 0.03), (sk.NEWTON, 0.004)])
+def test_two_fp64_flows_on_two_streams_equal_the_flows_alone(na, nb, mode, dt):
+    h, steps, launches = 0.25, 40, 4
+    pairs = [[on_gpu(field(n, h, 2 + k), h, 64)[:2] for k, n in enumerate((na, nb))] for _ in range(2)]
+    for lat, st in pairs[0]:
+        for _ in range(launches):
+            sk.flow_step(lat, dt, steps, mode, st)
+    graphs = [sk.FlowGraph(lat, st, dt, steps, mode) for lat, st in pairs[1]]
+    torch.cuda.synchronize()
+    for _ in range(launches):
+        for g in graphs:
+            with torch.cuda.stream(g.stream):  # each graph after its own last launch only
+                g.launch()
+    torch.cuda.synchronize()
+    for (_, alone), (_, both) in zip(*pairs):
+        rep = both.report()
+        assert rep == alone.report() and rep["steps"] == steps * launches and rep["status"] == 0
+        assert torch.equal(alone.phi, both.phi) and torch.equal(alone.vel, both.vel)
+    for g in graphs:
+        g.close()
+
+
 @pytest.mark.parametrize("n", SIZES + [(6, 40, 52)])
 @pytest.mark.parametrize("prec", [64, 32])
 def test_load_field_gives_the_same_state_from_every_source(n, prec):
