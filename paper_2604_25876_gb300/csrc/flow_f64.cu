@@ -635,6 +635,33 @@ template <bool EXT, int TZ> static cudaError_t launch_shape(F64Params &p, int st
     return cudaSuccess;
 }
 
+// SMs that kernels on stream s run on: a green context's share, else the
+// device's.  A cooperative launch of more CTAs than fit on them is refused.
+static cudaError_t stream_sms(cudaStream_t s, int *sms)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    static const auto entry = [](const char *name) -> void * {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        return cudaGetDriverEntryPointByVersion(name, &fn, 12040, cudaEnableDefault, &q) == cudaSuccess &&
+                       q == cudaDriverEntryPointSuccess
+                   ? fn
+                   : nullptr;
+    };
+    static const auto green_of = reinterpret_cast<PFN_cuStreamGetGreenCtx_v12040>(entry("cuStreamGetGreenCtx"));
+    static const auto resource =
+        reinterpret_cast<PFN_cuGreenCtxGetDevResource_v12040>(entry("cuGreenCtxGetDevResource"));
+    CUgreenCtx green = nullptr;
+    CUdevResource r;
+    if (green_of && resource && green_of(s, &green) == CUDA_SUCCESS && green &&
+        resource(green, &r, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS && r.sm.smCount > 0)
+        *sms = std::min(*sms, (int)r.sm.smCount);
+    return cudaSuccess;
+}
+
 cudaError_t launch_steps_f64(const skyrme_lattice &lat, const FlowArgs &a, int steps, cudaStream_t s)
 {
     F64Params p = {};
@@ -667,9 +694,8 @@ cudaError_t launch_steps_f64(const skyrme_lattice &lat, const FlowArgs &a, int s
                                    4.0 * B * B, 4.0 * B * B, a.c6 * k2 * k2 * k2, 0.0};
     for (int q = 0; q < kSums64; ++q) p.scale[q] = scale[q];
     p.h3 = a.h * a.h * a.h;
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int sms = 0;
+    const cudaError_t e = stream_sms(s, &sms);
     if (e != cudaSuccess) return e;
     // the column that pads the lattice less (4 x 8 forms twice the halo: 1%)
     const long long iy = p.n1 - 4, iz = p.n2 - 4;

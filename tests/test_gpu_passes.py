@@ -1,6 +1,8 @@
 """The passes over a whole field (energy, observables, render) at the sizes
 where their work splits have edges: lattices smaller than a tile or a chunk of
 planes, ragged sides, rows and planes one past a block, both z tiles."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -288,6 +290,53 @@ def test_two_fp64_flows_on_two_streams_equal_the_flows_alone(na, nb, mode, dt):
         assert torch.equal(alone.phi, both.phi) and torch.equal(alone.vel, both.vel)
     for g in graphs:
         g.close()
+
+
+def green_stream(sms):
+    """A stream that owns about ``sms`` of the device's SMs, and how many it
+    got (the driver's green contexts; its resource records are 144 bytes)."""
+    cu = ctypes.CDLL("libcuda.so.1")
+    if not hasattr(cu, "cuGreenCtxStreamCreate"):
+        pytest.skip("the driver has no green contexts")
+    torch.cuda.init()
+    device, part, rest = (ctypes.create_string_buffer(1024) for _ in range(3))
+    desc, ctx, stream = ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_void_p()
+    count = ctypes.c_uint(1)
+    for rc in (cu.cuDeviceGetDevResource(0, device, 1),
+               cu.cuDevSmResourceSplitByCount(part, ctypes.byref(count), device, rest, 0, sms),
+               cu.cuDevResourceGenerateDesc(ctypes.byref(desc), part, 1),
+               cu.cuGreenCtxCreate(ctypes.byref(ctx), desc, 0, 1),
+               cu.cuGreenCtxStreamCreate(ctypes.byref(stream), ctx, 1, 0)):
+        assert rc == 0
+    got = int.from_bytes(part.raw[96:100], "little")
+    return cu, ctx, torch.cuda.ExternalStream(stream.value), got
+
+
+# a stream that owns part of the SMs: launches that wait inside have to fit there
+@pytest.mark.parametrize("mode,dt", [(sk.ARRESTED, 0.03), (sk.NEWTON, 0.004)])
+@pytest.mark.parametrize("n", [(24, 48, 48), (70, 66, 68)])
+def test_fp64_flow_on_a_stream_of_a_green_context(n, mode, dt):
+    cu, ctx, s, sms = green_stream(32)
+    assert 0 < sms < torch.cuda.get_device_properties(0).multi_processor_count
+    h, steps = 0.25, 20
+    lat, a, phi = on_gpu(field(n, h, 2), h, 64)
+    _, b, _ = on_gpu(phi, h, 64)
+    _, c, _ = on_gpu(phi, h, 64)
+    torch.cuda.synchronize()
+    ra, rb = sk.flow_step(lat, dt, steps, mode, a), sk.flow_step(lat, dt, steps, mode, b, stream=s)
+    g = sk.FlowGraph(lat, c, dt, steps, mode, stream=s)
+    with torch.cuda.stream(s):
+        g.launch()
+    s.synchronize()
+    g.close()
+    # the sums run over other shares of the lattice (rounding: 1e4 terms), the
+    # sites' arithmetic is the same
+    for r in (rb, c.report()):
+        assert (r["steps"], r["arrests"], r["status"]) == (steps, ra["arrests"], 0)
+        assert r["E"] == pytest.approx(ra["E"], rel=1e-12)
+    assert torch.equal(a.phi, b.phi) and torch.equal(a.phi, c.phi)
+    assert torch.equal(a.vel, b.vel) and torch.equal(a.vel, c.vel)
+    assert cu.cuStreamDestroy_v2(ctypes.c_void_p(s.cuda_stream)) == 0 and cu.cuGreenCtxDestroy(ctx) == 0
 
 
 @pytest.mark.parametrize("n", SIZES + [(6, 40, 52)])
