@@ -149,7 +149,7 @@ skyrme_status skyrme_load_field(const skyrme_lattice *lat, skyrme_state *st, voi
  * alignment of phi), which is read once and must stay valid until the call's
  * work on `stream` is done: it saves the caller's copy into phi[0].
  * SKYRME_EINVAL when src is null or misaligned or overlaps the state's
- * buffers. */
+ * buffers (its scratch too). */
 skyrme_status skyrme_load_field_from(const skyrme_lattice *lat, skyrme_state *st, const void *src,
                                      void *stream);
 

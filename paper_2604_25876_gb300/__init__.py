@@ -393,7 +393,7 @@ def _loadable(lat: Lattice, st: State, t) -> bool:
         return False
     site, a = 4 * t.element_size(), t.data_ptr()
     b = a + t.numel() * t.element_size()
-    for buf in (st.phi, st.vel):
+    for buf in (st.phi, st.vel, st.scratch):
         lo = buf.data_ptr()
         if a < lo + buf.numel() * buf.element_size() and lo < b:
             return False

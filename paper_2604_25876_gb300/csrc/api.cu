@@ -292,9 +292,10 @@ skyrme_status skyrme_load_field_from(const skyrme_lattice *lat, skyrme_state *st
     const size_t align = site_bytes(*lat);
     if (!src || ((uintptr_t)src % align)) return SKYRME_EINVAL;
     const uintptr_t bytes = (uintptr_t)lat->n[0] * lat->n[1] * lat->n[2] * align;
-    for (int i = 0; i < 4; ++i) {
-        const uintptr_t b = (uintptr_t)(i < 2 ? st->phi[i] : st->vel[i - 2]), f = (uintptr_t)src;
-        if (f < b + bytes && b < f + bytes) return SKYRME_EINVAL;
+    const void *own[5] = {st->phi[0], st->phi[1], st->vel[0], st->vel[1], st->scratch};
+    for (int i = 0; i < 5; ++i) {
+        const uintptr_t b = (uintptr_t)own[i], f = (uintptr_t)src, len = i < 4 ? bytes : st->scratch_bytes;
+        if (f < b + len && b < f + bytes) return SKYRME_EINVAL;
     }
     CKDEV(state_on_device(st));
     CKDEV(on_current_device(&src, 1));

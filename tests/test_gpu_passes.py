@@ -382,3 +382,25 @@ def test_load_field_from_rejects_null_misaligned_and_overlapping_sources():
     assert call(st.phi[0].data_ptr() + 16) == 1 and call(st.vel[1].data_ptr()) == 1
     assert call(f.data_ptr() + 16) == 0
     torch.cuda.synchronize()
+
+
+# the load rewrites the control block while it reads its source, so a field in
+# the state's scratch (where the control block is) goes through a copy
+@pytest.mark.parametrize("prec", [64, 32])
+@pytest.mark.parametrize("offset", [0, 8192])
+def test_a_field_in_the_scratch_is_not_read_in_place(prec, offset):
+    n = (6, 7, 8)
+    lat = sk.Lattice(n, 0.25, 1.0, prec)
+    st = sk.State(lat, DEV)
+    t = torch.from_numpy(field(n, 0.25, 3)).to(DEV, lat.dtype)
+    nbytes = t.numel() * t.element_size()
+    src = st.scratch[offset:offset + nbytes].view(lat.dtype).view(t.shape)
+    cl, cs = lat.c(), st.c()
+    rc = sk.load().skyrme_load_field_from(ctypes.byref(cl), ctypes.byref(cs),
+                                          ctypes.c_void_p(src.data_ptr()), None)
+    assert rc == 1
+    src.copy_(t)
+    sk.load_field(lat, st, src)
+    ref = torch.from_numpy(oracle.apply_vacuum_boundary(t.double().cpu().numpy())).to(DEV, lat.dtype)
+    assert torch.equal(st.phi[0], ref) and torch.equal(st.phi[1], ref) and not st.vel.any().item()
+    assert sk.read_report(lat, st)["steps"] == 0
