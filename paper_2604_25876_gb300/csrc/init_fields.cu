@@ -207,14 +207,25 @@ __global__ void k_profile_table(double2 *table, int base, double scale)
     for (int k = 0; k < N; ++k) table[i * N + k] = make_double2(C[k], S[k]);
 }
 
-// C and S at q = r^2, directly.
+// A scale whose reciprocal and products are far from the ends of the range.
+static bool ordinary_scale(double scale) { return scale > 1e-100 && scale < 1e100; }
+
+// C and S at q = r^2, directly.  inv_scale: 0 unless the scale is an ordinary one.
 __device__ __forceinline__ void profile_direct(double q, double scale, double inv_scale, double &c, double &s)
 {
-    const double inv = q > 0.0 ? rsqrt(q) : 0.0;
-    double r = q * inv;
-    r = ::fma(0.5 * inv, ::fma(-r, r, q), r);
-    double rho = r * inv_scale;
-    rho = ::fma(::fma(-rho, scale, r), inv_scale, rho);
+    double inv, rho;
+    // (the test is on the integer pipe: 2^-600 <= q < 2^600)
+    if ((unsigned)__double2hiint(q) - 0x1a700000u < 0x4b000000u && inv_scale != 0.0) {
+        inv = rsqrt(q);
+        double r = q * inv;
+        r = ::fma(0.5 * inv, ::fma(-r, r, q), r);
+        rho = r * inv_scale;
+        rho = ::fma(::fma(-rho, scale, r), inv_scale, rho);
+    } else {  // r = 0, or a step of the above could overflow
+        const double r = sqrt(q);
+        inv = r > 0.0 ? 1.0 / r : 0.0;
+        rho = r / scale;
+    }
     sincospi(exp(-rho), &s, &c);
     s *= inv;
 }
@@ -228,7 +239,7 @@ __device__ __forceinline__ void product_site(const ProductArgs &a, double cx, do
     double fwd[4], rev[4];
     for (int k = 0; k < a.K; ++k) {
         const Constituent &c = a.c[k];
-        const double dx = cx - c.pos[0], dy = cy - c.pos[1], dz = cz - c.pos[2];
+        double dx = cx - c.pos[0], dy = cy - c.pos[1], dz = cz - c.pos[2];
         const double q = dx * dx + dy * dy + dz * dz;
         double cf, sf;
         const int j = (__double2hiint(q) >> 15) - a.base;
@@ -245,6 +256,8 @@ __device__ __forceinline__ void product_site(const ProductArgs &a, double cx, do
             }
         } else {
             profile_direct(q, a.scale, a.inv_scale, cf, sf);
+            // r^2 overflows: sf = 0, and the rotation's sums may overflow too
+            if (__double2hiint(q) == 0x7ff00000) dx = dy = dz = 0.0;
         }
         const double u[4] = {cf * c.norm, sf * (c.rot[0][0] * dx + c.rot[0][1] * dy + c.rot[0][2] * dz),
                              sf * (c.rot[1][0] * dx + c.rot[1][1] * dy + c.rot[1][2] * dz),
@@ -765,7 +778,7 @@ static int grid_for(size_t total)
 static bool pairs_apply(const skyrme_lattice &lat, const ProductArgs &pa)
 {
     const double total = (double)lat.n[0] * lat.n[1] * lat.n[2];
-    if (lat.n[2] < 24 || total >= 4.2e9 || total * sizeof(float4) < (double)kPairTableBytes) return false;
+    if (pa.inv_scale == 0.0 || lat.n[2] < 24 || total >= 4.2e9 || total * sizeof(float4) < (double)kPairTableBytes) return false;
     double inside = 1.0;
     for (int j = 0; j < 3; ++j) {
         double reach = 0.0;
@@ -813,7 +826,7 @@ static cudaError_t seed_impl(const skyrme_lattice &lat, const skyrme_seed &sd, c
         ProductArgs pa;
         pa.K = sd.B;
         pa.scale = sd.profile_scale;
-        pa.inv_scale = 1.0 / sd.profile_scale;
+        pa.inv_scale = ordinary_scale(sd.profile_scale) ? 1.0 / sd.profile_scale : 0.0;
         pa.table = nullptr;
         pa.base = 0;
         for (int k = 0; k < sd.B; ++k) {
@@ -839,7 +852,7 @@ static cudaError_t seed_impl(const skyrme_lattice &lat, const skyrme_seed &sd, c
         // The table costs a launch of 26 us and saves 30 instructions per site
         // and constituent (48 us per million of them); it needs the scratch
         // behind the control block and an ordinary scale.
-        if (work >= 1e6 && scratch_bytes >= kProfileTableBytes && sd.profile_scale > 1e-100 && sd.profile_scale < 1e100) {
+        if (work >= 1e6 && scratch_bytes >= kProfileTableBytes && ordinary_scale(sd.profile_scale)) {
             pa.base = profile_base(sd.profile_scale);
             double2 *table = reinterpret_cast<double2 *>(a.step_parts);
             k_profile_table<<<(kProfileIntervals + 31) / 32, 32, 0, s>>>(table, pa.base, pa.scale);

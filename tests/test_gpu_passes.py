@@ -168,6 +168,32 @@ def test_product_seed_matches_oracle(n, h, K, scale, prec, sym):
     assert sk.read_report(lat, st)["steps"] == 0
 
 
+# positions so far off that r^2 overflows (such a constituent is the vacuum),
+# scales whose reciprocal overflows or is 0, and scales at the ends of the
+# table's range; on both sides of the sizes from which the table and the
+# double-float kernel are taken
+@pytest.mark.parametrize("n,K", [((7, 9, 26), 2), ((64, 64, 64), 5)])
+@pytest.mark.parametrize("far,scale", [(1e160, 1.0), (-3e300, 1.0), (0.0, 1e-309), (0.0, 1e-305),
+                                       (0.0, 1e-90), (0.0, 1e90), (0.0, 1e300), (0.0, np.inf)])
+@pytest.mark.parametrize("prec", [64, 32])
+@pytest.mark.parametrize("sym", [True, False])
+def test_product_seed_at_the_ends_of_the_number_range(n, K, far, scale, prec, sym):
+    rng = np.random.default_rng(K)
+    pos = rng.uniform(-1.0, 1.0, size=(K, 3))
+    pos[0] = [(n[a] // 2 - 0.5 * (n[a] - 1)) * 0.25 for a in range(3)]  # r = 0 at a site
+    pos[1] += [far, 0.0, -far]
+    q = rng.normal(size=(K, 4))
+    q /= np.linalg.norm(q, axis=1, keepdims=True)
+    lat = sk.Lattice(n, 0.25, 1.0, prec)
+    st = sk.State(lat, DEV)
+    sk.init_field(lat, sk.Seed.product(pos, q, scale, sym), st)
+    ref = oracle.seed_product(n, 0.25, pos, q, scale, sym)
+    assert np.isfinite(ref).all()
+    got = st.phi[0].double().cpu().numpy()
+    # as above: a few eps per constituent, or the FP32 rounding
+    assert np.max(np.abs(got - ref)) <= (1e-12 if prec == 64 else 1.2e-7)
+
+
 # the double-float kernel: rows of 24 sites, of one and a bit of a warp, a
 # constituent on a site, radii on both sides of the table's ends (rho = 1/64
 # and 32), many constituents, a coarse and a fine lattice
