@@ -325,11 +325,13 @@ __global__ void __launch_bounds__(256) k_seed_product(vec4_t<T> *phi0, vec4_t<T>
 // The field of an FP32 state is rounded to 24 bits at the end, and the FP32
 // pipe issues 64 times the FP64 pipe's instructions.  k_seed_product_f32
 // evaluates the ansatz in unevaluated sums hi + lo of two floats (error-free
-// products by FMA, Knuth's and Dekker's sums), with a bound on the error beside
-// it, and stores hi where no value within the bound rounds to another float:
-// it is then the rounding of the exact field.  The sites where the bound does
-// not decide (one in 150 with eight constituents), and those where a profile is
-// outside the table, are collected per warp and evaluated in FP64, 32 at a time.
+// products by FMA, Knuth's and Dekker's sums), with a margin for the error beside
+// it, and stores hi where no value within the margin rounds to another float.
+// The margin is measured, not proven (kPairEps); should an error ever exceed it,
+// the value stored is at most one ulp from the rounding of the exact one.  The
+// sites where the margin does not decide (one in 150 with eight constituents),
+// and those where a profile is outside the table, are collected per warp and
+// evaluated in FP64, 32 at a time.
 //
 // Positions are in units of the profile's scale.  A warp takes 32 sites along
 // z; the rotated offsets R_k (x - x_k) of its middle come from FP64 once per
@@ -352,10 +354,14 @@ constexpr int kPairIntervals = kPairOctaves * kPairPerOctave;
 constexpr int kPairBase = (127 - 12) * kPairPerOctave;
 constexpr int kPairVecs = 5;  // float4 per interval: (C, S) pairs hi, lo of degrees 0 to 2, then 3 to 6
 constexpr size_t kPairTableBytes = (size_t)kPairIntervals * kPairVecs * sizeof(float4);
-// The bounds err[] below: the scalar component's error against 1, the others'
-// against the sum of the constituents' pion sizes.  Over lattice spacings of 0.02
-// to 2 scales and 1 to 64 constituents the largest error met was 0.22 of them.
-constexpr float kPairEps = 0x1p-40f;
+// The margins err[] below: a scalar component's error goes with the number of
+// products and with the vector errors that each product hands it, a vector
+// component's with P, the sum of the constituents' pion sizes; how these grow was
+// taken from the arithmetic, their factors from comparisons with FP64.  Over
+// lattice spacings of 0.001 to 2.7 scales (pairs_apply) and 1 to 64 constituents,
+// spread out, in one place, alike and with one dominating, the largest error met
+// was 0.20 of them (0.56 without the P^2 term, with 64 constituents at 0.02).
+constexpr float kPairEps = 0x1p-40f, kPairCross = 1.f / 64;
 
 __global__ void k_pair_table(float4 *table)
 {
@@ -428,14 +434,14 @@ __device__ __forceinline__ void mul_pairs(Pairs4 &x, const Pairs4 &y, const Pair
     x = r;
 }
 
-// The ansatz at a lane's site: val[] its components hi + lo, err[] bounds on the
-// errors of the scalar component and of the others.  ob[3 k + i]: component i
+// The ansatz at a lane's site: val[] its components hi + lo, err[] margins for
+// their errors.  ob[3 k + i]: component i
 // of the rotated offset of constituent k from the warp's middle (hi, lo) and
 // its increment along z (hi, lo); zl: the lane's site from the middle.  False
 // where a profile is outside the table.
 template <bool SYM>
 __device__ __forceinline__ bool product_pairs(const float4 *ob, int K, const float4 *__restrict__ table, float zl,
-                                              float hs, DF (&val)[4], float (&err)[2])
+                                              float hs, DF (&val)[4], float (&err)[4])
 {
     Pairs4 x;  // U_1 ... U_k and the conjugate of U_k ... U_1, which is conj(U_1) ... conj(U_k)
     float P = 0.f;
@@ -494,12 +500,15 @@ __device__ __forceinline__ bool product_pairs(const float4 *ob, int K, const flo
             mul_pairs(x, y, n, bc(3.f), bc(big));
         }
     }
-    const float eps = kPairEps * __fmaf_rn(4.f, hs, 1.f), eps0 = eps * (1.f + (float)K),
-                eps1 = eps * __fmaf_rn(0.0625f, (float)K, 1.f);
+    // the scalar's margin grows with P^2 too: each product hands it the vector's error
+    const float eps = kPairEps * __fmaf_rn(4.f, hs, 1.f), e0 = eps * (1.f + (float)K + kPairCross * P * P),
+                e1 = eps * __fmaf_rn(0.0625f, (float)K, 1.f) * P;
     if (!SYM) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) val[i] = quick_two_sum(x.h[i].x, x.l[i].x);
-        err[0] = eps0, err[1] = eps1 * P;
+        for (int i = 0; i < 4; ++i) {
+            val[i] = quick_two_sum(x.h[i].x, x.l[i].x);
+            err[i] = i == 0 ? e0 : e1;
+        }
         return true;
     }
     // t = U_1 ... U_K + U_K ... U_1, divided by its norm
@@ -519,10 +528,14 @@ __device__ __forceinline__ bool product_pairs(const float4 *ob, int K, const flo
     const float be = __fmaf_rn(q.lo, a, __fmaf_rn(q.hi, ae, __fmaf_rn(q.hi, a, -b)));
     const float g = __fsub_rn(__fsub_rn(1.f, b), be);
     const DF y = {y0, __fmul_rn(__fmul_rn(y0, g), __fmaf_rn(0.375f, g, 0.5f))};
+    // (2 y0 >= 1: |t| <= 2)  A component's error, and what the others' do to it through the norm
+    const float y2 = 4.f * (y0 * y0);
 #pragma unroll
     for (int i = 0; i < 4; ++i) val[i] = df_mul(t[i], y);
-    const float y2 = 4.f * (y0 * y0);
-    err[0] = eps0 * y2, err[1] = eps1 * P * y2;
+    const float v0 = fabsf(val[0].hi), vs = fabsf(val[1].hi) + fabsf(val[2].hi) + fabsf(val[3].hi);
+    err[0] = y2 * __fmaf_rn(v0 * vs, e1, e0);
+#pragma unroll
+    for (int i = 1; i < 4; ++i) err[i] = y2 * __fmaf_rn(fabsf(val[i].hi), __fmaf_rn(vs, e1, v0 * e0), e1);
     return true;
 }
 
@@ -532,7 +545,7 @@ __device__ __forceinline__ double to_double(int i)
     return __hiloint2double(0x43300000, i ^ (int)0x80000000) - (0x1p52 + 0x1p31);
 }
 
-// The sites the bound left open, in FP64.
+// The sites the margin left open, in FP64.
 template <bool SYM>
 __device__ __noinline__ void product_open(const ProductArgs &a, float4 *phi0, float4 *phi1, unsigned s, int n0, int n1,
                                           int n2, double h)
@@ -590,14 +603,13 @@ __global__ void __launch_bounds__(32 * kPairWarps, 2)
             __syncwarp();
             if (z >= 2 && z <= n2 - 3) {
                 DF v[4];
-                float err[2];
+                float err[4];
                 sure = product_pairs<SYM>(s_ob[warp], a.K, table, (float)(lane - 16), (float)hs, v, err);
                 if (sure) {
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        const float e = err[i > 0];
-                        sure = sure && __fadd_rn(v[i].hi, __fadd_rn(v[i].lo, e)) == v[i].hi &&
-                               __fadd_rn(v[i].hi, __fsub_rn(v[i].lo, e)) == v[i].hi;
+                        sure = sure && __fadd_rn(v[i].hi, __fadd_rn(v[i].lo, err[i])) == v[i].hi &&
+                               __fadd_rn(v[i].hi, __fsub_rn(v[i].lo, err[i])) == v[i].hi;
                     }
                     out = make_float4(v[0].hi, v[1].hi, v[2].hi, v[3].hi);
                 }
@@ -770,8 +782,9 @@ static int grid_for(size_t total)
 }
 
 // Whether the double-float kernel takes the ansatz: unit orientations, rows that
-// fill a warp, 32-bit indices, offsets small enough for their rounding, and a
-// lattice that lies largely inside the table (32 scales from a constituent):
+// fill a warp, 32-bit indices, a spacing at which the error was measured (coarser
+// ones than 2.7 scales fail the last condition), offsets small enough for their
+// rounding, and a lattice that lies largely inside the table (32 scales from a constituent):
 // outside, the attempt costs 7% on top of the FP64 evaluation.  At 128^3 with 4
 // constituents, FP64 and double-float: 1.69 and 1.82 ms with nearly every site
 // outside, 1.73 and 1.74 ms with a box of +-64 scales (the estimate is then 0.08).
@@ -779,6 +792,8 @@ static bool pairs_apply(const skyrme_lattice &lat, const ProductArgs &pa)
 {
     const double total = (double)lat.n[0] * lat.n[1] * lat.n[2];
     if (pa.inv_scale == 0.0 || lat.n[2] < 24 || total >= 4.2e9 || total * sizeof(float4) < (double)kPairTableBytes) return false;
+    const double hs = lat.h * pa.inv_scale;
+    if (!(hs >= 0.001 && hs <= 2.75)) return false;
     double inside = 1.0;
     for (int j = 0; j < 3; ++j) {
         double reach = 0.0;

@@ -225,6 +225,53 @@ def test_large_fp32_product_seed_is_the_rounded_fp64_seed(n, h, K, scale, sym):
     assert torch.all((phi[32] - ref).abs()[off] <= 1.3e-7 * ref.abs()[off])
 
 
+def captured_nodes(call):
+    """How many kernels, copies and memsets ``call`` puts on its stream."""
+    cu = ctypes.CDLL("libcuda.so.1")
+    graph, s = torch.cuda.CUDAGraph(keep_graph=True), torch.cuda.Stream(DEV)
+    with torch.cuda.graph(graph, stream=s):
+        call()
+    h, n = ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t()
+    assert cu.cuGraphGetNodes(h, None, ctypes.byref(n)) == 0
+    nodes, kind, count = (ctypes.c_void_p * n.value)(), ctypes.c_int(), [0, 0, 0]
+    assert cu.cuGraphGetNodes(h, nodes, ctypes.byref(n)) == 0
+    for node in nodes:
+        assert cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        count[kind.value] += 1
+    return dict(zip(("kernels", "copies", "memsets"), count))
+
+
+# The double-float kernel's margins, where products hand the scalar component the
+# most error and where one constituent's vector is most of the site's; and only
+# spacings at which the margins were measured take it (it clears its table).
+@pytest.mark.parametrize("hs,radius,dominant,pairs", [(0.02, 0.3, False, True), (0.1, 0.0, False, True),
+                                                      (0.1, 5.0, True, True), (0.0009, 0.01, False, False),
+                                                      (0.001, 0.01, False, True)])
+@pytest.mark.parametrize("sym", [True, False])
+def test_fp32_product_seed_of_many_constituents(hs, radius, dominant, pairs, sym):
+    n, scale, K = (40, 44, 45), 1.6, 64
+    rng = np.random.default_rng(11)
+    pos = rng.uniform(-1.0, 1.0, size=(K, 3)) * radius * scale
+    if dominant:
+        pos = np.sign(pos) * (0.6 * radius * scale + 0.4 * np.abs(pos))
+        pos[K // 2] = [0.01, 0.0, -0.02]
+    q = rng.normal(size=(K, 4))
+    q /= np.linalg.norm(q, axis=1, keepdims=True)
+    phi = {}
+    for prec in (32, 64):
+        lat = sk.Lattice(n, hs * scale, 1.0, prec)
+        st, seed = sk.State(lat, DEV), sk.Seed.product(pos, q, scale, sym)
+        if prec == 32:
+            assert captured_nodes(lambda: sk.init_field(lat, seed, st))["memsets"] == (1 if pairs else 0)
+        sk.init_field(lat, seed, st)
+        phi[prec] = st.phi[0].cpu()
+    # as above: 1e-14 / 6e-8 of 3e5 values, one ulp each
+    ref = phi[64].float()
+    off = phi[32] != ref
+    assert int(off.sum()) <= 4
+    assert torch.all((phi[32] - ref).abs()[off] <= 1.3e-7 * ref.abs()[off])
+
+
 # the FP64 step's columns (2 x 16 or 4 x 8), runs and shares: lattices of fewer
 # units than warps, runs that cross columns, both column shapes, long runs
 @pytest.mark.parametrize("n", SIZES + [(33, 48, 48), (200, 14, 18)])
