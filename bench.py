@@ -131,10 +131,10 @@ def step_kernel_key(wl, prec):
 def step_launches(wl, prec, steps):
     """Kernel launches of a graph of ``steps`` ARRESTED iterations: one each for
     the FP32 streaming step, and for the FP64 step one for as many iterations as
-    update 2^22 sites (both correct their own mispredictions); with a fix-up
-    check each for the FP32 tile step."""
+    update 2^22 sites, up to 128 (both correct their own mispredictions); with a
+    fix-up check each for the FP32 tile step."""
     if prec == 64:
-        return math.ceil(steps / max(1, min(steps, (1 << 22) // wl.interior_sites)))
+        return math.ceil(steps / max(1, min(steps, 128, (1 << 22) // wl.interior_sites)))
     return steps if wl.streaming else 2 * steps
 
 

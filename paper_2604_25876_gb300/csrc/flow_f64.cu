@@ -27,7 +27,7 @@
 //  * Units per warp decide the time of a small lattice, so the launch takes 8,
 //    6 or 4 warps per SM, whichever leaves the busiest SM less to do
 //    (plan_warps).
-//  * A launch runs several steps of a small lattice (kLaunchSites): every CTA
+//  * A launch runs several steps of a small lattice (kLaunchSites, kLaunchSteps): every CTA
 //    waits for the decision and goes on to the next step, over one more barrier
 //    when sites were corrected.  One step per launch and now, us per step in a
 //    graph and on a stream: 24 x 26 x 28 26.9 and 29.2 -> 25.7 and 26.0, 48^3
@@ -60,7 +60,8 @@ namespace skyrme {
 constexpr int kMaxWarps = 8;    // per CTA, one CTA per SM
 constexpr int kMaxShare = 160 * kMaxWarps;  // warps of a launch
 constexpr int kPlaneSlots = 4;  // planes x .. x + 2 of the centre, and the next one arriving
-constexpr double kLaunchSites = 1 << 22;  // site updates of a launch of several steps
+constexpr double kLaunchSites = 1 << 22;  // site updates of a launch of several steps,
+constexpr int kLaunchSteps = 128;         // and its steps, at most
 constexpr int kSums64 = 8;      // e2, e4, potential, det, |F|^2, max |F|^2, e6, (unused)
 
 struct F64Params {
@@ -676,10 +677,12 @@ cudaError_t launch_steps_f64(const skyrme_lattice &lat, const FlowArgs &a, int s
     p.nix = p.n0 - 4;
     p.mode = a.mode;
     p.fuse_fix = a.mode == SKYRME_ARRESTED && !a.slab_rec;
-    // A launch runs as many steps as update kLaunchSites sites, about 3 ms: more
-    // save nothing, and other streams' kernels start between launches.
+    // A launch runs as many steps as update kLaunchSites sites, but kLaunchSteps at
+    // most (a step of the smallest lattices is all fixed costs, 20 us): 2 to 5 ms.
+    // More save nothing, and other streams' kernels start between launches.
     const double sites = (double)(p.n0 - 4) * (p.n1 - 4) * (p.n2 - 4);
-    p.steps = a.slab_rec ? 1 : (int)std::max(1.0, std::min((double)steps, kLaunchSites / sites));
+    const double most = std::min((double)kLaunchSteps, kLaunchSites / sites);
+    p.steps = a.slab_rec ? 1 : (int)std::max(1.0, std::min((double)steps, most));
     const double k1 = 1.0 / (12.0 * a.h), k2 = k1 * k1, B = 12.0 * k2 * k2;
     p.dt = a.dt;
     p.dt2 = 2.0 * a.dt * B;

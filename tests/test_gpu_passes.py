@@ -6,8 +6,10 @@ import ctypes
 import numpy as np
 import pytest
 
+import bench
 import oracle
 import paper_2604_25876_gb300 as sk
+import workloads
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -337,6 +339,27 @@ def test_fp64_corrections_in_a_launch_equal_single_steps(n, model, dt, entry):
     assert a == b and b["steps"] == steps and b["status"] == 0
     assert b["fixups"] > 1
     assert torch.equal(one.phi, many.phi) and torch.equal(one.vel, many.vel)
+
+
+# as many steps to a launch as update 2^22 sites, and 128 at most
+@pytest.mark.parametrize("n,steps,launches", [((8, 8, 8), 300, 3), ((24, 26, 28), 129, 2), ((24, 26, 28), 128, 1),
+                                              ((48, 48, 48), 100, 3), ((170, 160, 180), 3, 3)])
+@pytest.mark.parametrize("mode", [sk.ARRESTED, sk.NEWTON])
+def test_fp64_steps_in_a_launch_are_capped(n, steps, launches, mode):
+    lat = sk.Lattice(n, 0.25, 1.0, 64)
+    st = sk.State(lat, DEV)
+    sk.init_field(lat, sk.Seed.rational_map(1, 0.5), st)
+    cl, cs = lat.c(), st.c()
+
+    def call():
+        rc = sk.load().skyrme_flow_step(ctypes.byref(cl), 0.004, steps, mode, ctypes.byref(cs), None,
+                                        ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+        assert rc == 0
+    call()  # (a captured launch is not the first)
+    torch.cuda.synchronize()
+    assert captured_nodes(call) == {"kernels": launches, "copies": 0, "memsets": 0}
+    wl = workloads.Workload("box", n, 0.25, 1.0, steps, 64, None, 0.004)
+    assert bench.step_launches(wl, 64, steps) == launches
 
 
 # launches that wait inside (for the arrest decision, for the next step) on two
