@@ -335,6 +335,15 @@ class Seed:
         return s, (pos, q)  # keep host arrays alive during the call
 
 
+def _pair(buf) -> _VoidP2:
+    """The addresses of buf[0] and buf[1]: in a tensor of two buffers the second
+    lies one stride behind the first (indexing would make a tensor)."""
+    if isinstance(buf, _torch().Tensor) and buf.shape[0] > 1:
+        p = buf.data_ptr()
+        return _VoidP2(p, p + buf.stride()[0] * buf.itemsize)
+    return _VoidP2(buf[0].data_ptr(), buf[1].data_ptr())
+
+
 class State:
     """Device buffers of one lattice: two field and two velocity buffers
     (torch tensors of shape (2, Nx, Ny, Nz, 4)) and the scratch block."""
@@ -349,12 +358,8 @@ class State:
         self.scratch = torch.zeros(lat.scratch_bytes(), dtype=torch.uint8, device=self.device)
 
     def c(self) -> c_state:
-        # phi[1] lies one stride behind phi[0] (indexing would make a tensor)
-        phi, vel, scratch = self.phi, self.vel, self.scratch
-        p, v = phi.data_ptr(), vel.data_ptr()
-        return c_state(_VoidP2(p, p + phi.stride(0) * phi.element_size()),
-                       _VoidP2(v, v + vel.stride(0) * vel.element_size()),
-                       scratch.data_ptr(), scratch.numel())
+        scratch = self.scratch
+        return c_state(_pair(self.phi), _pair(self.vel), scratch.data_ptr(), scratch.numel())
 
     def report(self, stream=None) -> dict:
         return read_report(self.lat, self, stream)
@@ -382,20 +387,22 @@ def init_field(lat: Lattice, seed: Seed, st: State, stream=None):
     del keep
 
 
-def _loadable(lat: Lattice, st: State, t) -> bool:
+def _loadable(lat: Lattice, st: State, cs: c_state, t) -> bool:
     """Whether the load kernel can read the tensor where it is: a plain
     contiguous tensor of the state's device, precision and shape, aligned to a
     site and apart from the state's buffers."""
     torch = _torch()
+    if not isinstance(st.phi, torch.Tensor) or not isinstance(st.vel, torch.Tensor):
+        return False
     if type(t) is not torch.Tensor or not t.is_cuda or t.device != st.phi.device or \
             t.dtype != lat.dtype or t.shape != st.phi.shape[1:] or not t.is_contiguous() or \
             t.requires_grad or t.is_neg() or t.numel() == 0:
         return False
-    site, a = 4 * t.element_size(), t.data_ptr()
-    b = a + t.numel() * t.element_size()
-    for buf in (st.phi, st.vel, st.scratch):
-        lo = buf.data_ptr()
-        if a < lo + buf.numel() * buf.element_size() and lo < b:
+    site, size, a = 4 * t.element_size(), t.numel() * t.element_size(), t.data_ptr()
+    if a < cs.scratch + cs.scratch_bytes and cs.scratch < a + size:
+        return False
+    for p in (cs.phi[0], cs.phi[1], cs.vel[0], cs.vel[1]):
+        if a < p + size and p < a + size:
             return False
     return a % site == 0
 
@@ -406,7 +413,7 @@ def load_field(lat: Lattice, st: State, phi, stream=None):
     torch = _torch()
     t = torch.as_tensor(np.asarray(phi) if not isinstance(phi, torch.Tensor) else phi)
     cl, cs = lat.c(), st.c()
-    if stream is None and _loadable(lat, st, t):
+    if stream is None and _loadable(lat, st, cs, t):
         # read by the load kernel itself, on the current stream as the copy is
         _check(_on(st.device).skyrme_load_field_from(ctypes.byref(cl), ctypes.byref(cs),
                                                      ctypes.c_void_p(t.data_ptr()),

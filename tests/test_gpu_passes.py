@@ -462,6 +462,15 @@ def test_load_field_gives_the_same_state_from_every_source(n, prec):
         assert not st.vel.any().item()
         rep = sk.read_report(lat, st)
         assert rep["steps"] == 0 and rep["cur"] == 0 and rep["status"] == 0
+    st, wide = sk.State(lat, DEV), torch.zeros((4,) + t.shape, dtype=lat.dtype, device=DEV)
+    st.phi = wide[::2]  # buffers apart, the source the second of them
+    wide[2].copy_(t)
+    sk.load_field(lat, st, wide[2])
+    assert torch.equal(wide[0], ref) and torch.equal(wide[2], ref) and not wide[1::2].any().item()
+    st = sk.State(lat, DEV)  # buffers of their own
+    st.phi, st.vel = [torch.empty_like(t) for _ in range(2)], [torch.empty_like(t) for _ in range(2)]
+    sk.load_field(lat, st, t)
+    assert torch.equal(st.phi[0], ref) and torch.equal(st.phi[1], ref)
     with pytest.raises(RuntimeError):  # shapes that do not broadcast stay refused
         sk.load_field(lat, sk.State(lat, DEV), t[1:])
 
