@@ -226,22 +226,36 @@ def source_code_only(text: str) -> str:
     return " ".join(text.split())
 
 
-def kernel_fingerprint(kernel_key: str):
-    """Hash of the code of a step kernel's sources: the FP32 streaming
-    kernel (keys step_f32_*) or the FP64 step (every other key), with
-    their shared header; comments and layout do not count."""
-    h = hashlib.sha256()
+def kernel_sources(kernel_key: str):
+    """The csrc files a step kernel's code comes from, headers included (read
+    from the sources' own include lines): the FP32 streaming kernel (keys
+    step_f32_*), or for every other key the FP64 step and the tile kernels
+    (gradient flows, and FP32 fields without a tensor-map encoder)."""
     csrc = os.path.join(ROOT, "paper_2604_25876_gb300", "csrc")
-    src = "flow_f32.cu" if kernel_key.startswith("step_f32_") else "flow_f64.cu"
-    for name in (src, "skyrme_device.cuh"):
+    names = ["flow_f32.cu"] if kernel_key.startswith("step_f32_") else ["flow_f64.cu", "flow_generic.cu"]
+    for name in names:  # (grows while it is read)
         with open(os.path.join(csrc, name), encoding="utf-8") as f:
+            for inc in re.findall(r'^\s*#\s*include\s+"([^"]+)"', f.read(), flags=re.M):
+                if inc not in names and os.path.exists(os.path.join(csrc, inc)):
+                    names.append(inc)
+    return [os.path.join(csrc, name) for name in names]
+
+
+def kernel_fingerprint(kernel_key: str):
+    """Hash of the code of a step kernel's sources (kernel_sources); comments
+    and layout do not count."""
+    h = hashlib.sha256()
+    for path in kernel_sources(kernel_key):
+        with open(path, encoding="utf-8") as f:
             h.update(source_code_only(f.read()).encode())
     return h.hexdigest()[:16]
 
 
 def recorded_traffic(kernel_key: str, per_launch_sites: int):
-    """DRAM bytes per launch from the committed ncu summary, or None when the
-    kernel source changed since the counters were taken."""
+    """DRAM bytes of one iteration, launched by itself with cold caches, from
+    the committed ncu summary, or None when the kernel source changed since
+    the counters were taken.  (The FP64 step runs several iterations of a small
+    lattice in a launch; those after the first find it in L2.)"""
     path = os.path.join(ROOT, "profiles", "traffic.json")
     try:
         with open(path) as f:

@@ -3,6 +3,7 @@ kernel each workload runs on, the algorithmic figures its roofline uses, the
 lookup of recorded DRAM traffic, and the bounds that keep the bench short."""
 import json
 import os
+import shutil
 
 import pytest
 
@@ -70,6 +71,25 @@ def test_kernel_fingerprints_follow_the_kernel_sources():
     tile = bench.kernel_fingerprint("step_tile_f32_b4_sextic_128")
     assert tile == bench.kernel_fingerprint("step_f64_b1_hedgehog_48") and tile != f32
     assert len(f32) == 16 and int(f32, 16) >= 0
+
+
+@pytest.mark.parametrize("name,f32,f64", [("packed_f32.cuh", True, False), ("tma.cuh", True, True),
+                                          ("skyrme_device.cuh", True, True), ("flow_f32.cu", True, False),
+                                          ("flow_f64.cu", False, True), ("flow_generic.cu", False, True),
+                                          ("render.cu", False, False)])
+def test_a_kernel_fingerprint_covers_every_file_of_the_kernel(tmp_path, monkeypatch, name, f32, f64):
+    csrc = os.path.join("paper_2604_25876_gb300", "csrc")
+    shutil.copytree(os.path.join(ROOT, csrc), tmp_path / csrc)
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    keys = ("step_f32_b4_cubic_128", "step_f64_b1_hedgehog_48", "step_tile_f32_b4_sextic_128")
+    before = [bench.kernel_fingerprint(k) for k in keys]
+    with open(tmp_path / csrc / name, "a") as f:
+        f.write("// a comment\n")
+    assert [bench.kernel_fingerprint(k) for k in keys] == before
+    with open(tmp_path / csrc / name, "a") as f:
+        f.write("inline int one_more() { return 1; }\n")
+    changed = [a != b for a, b in zip(before, (bench.kernel_fingerprint(k) for k in keys))]
+    assert changed == [f32, f64, f64]
 
 
 def test_run_to_tolerance_leg_is_bounded():
