@@ -63,7 +63,7 @@ typedef enum { SKYRME_NEWTON = 0, SKYRME_ARRESTED = 1, SKYRME_GRADIENT = 2 } sky
  * SKYRME_EUNSUPPORTED, and so does the batched flow when c6 != 0 (batches
  * take the standard model and the potentials).  An FP32 flow runs on the
  * streaming FP32 kernel with any of the terms; an FP64 flow on the FP64 step
- * kernel. */
+ * kernel, and in GRADIENT mode on the tile kernel. */
 typedef struct {
     int n[3];       /* sites per axis (x slowest, z fastest); each >= 5 */
     double h;       /* lattice spacing, > 0, equal on every axis */

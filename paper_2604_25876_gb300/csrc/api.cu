@@ -316,8 +316,8 @@ static skyrme_status launch_iterations(const skyrme_lattice &lat, const FlowArgs
                                        cudaStream_t s)
 {
     // FP32: the streaming kernel (the standard model, the Section 7.8
-    // potentials, the sextic term); FP64: its own; FP32 without a tensor-map
-    // encoder: the tile kernel and the fix-up
+    // potentials, the sextic term); FP64: its own, but for gradient flows; those,
+    // and FP32 without a tensor-map encoder: the tile kernel (and the fix-up)
     if (fp32_streaming(lat)) {
         CK(launch_iterations_f32_fast(lat, a, nsteps, s), "step and fix-up kernels (fp32)");
         return SKYRME_OK;
@@ -328,9 +328,8 @@ static skyrme_status launch_iterations(const skyrme_lattice &lat, const FlowArgs
     }
     for (int k = 0; k < nsteps; ++k) {
         CK(launch_step(lat, a, s), "step kernel");
-        // the FP64 step corrects its own sites; an x-slab's fix-up follows the
-        // decision over all slabs
-        if (lat.precision == 32 && a.mode == SKYRME_ARRESTED && !a.slab_rec)
+        // (an x-slab's fix-up follows the decision over all slabs)
+        if (a.mode == SKYRME_ARRESTED && !a.slab_rec)
             CK(launch_fixup(lat, a, s), "fix-up kernel");
     }
     return SKYRME_OK;

@@ -67,6 +67,7 @@ bool lattice_ok(const skyrme_lattice *lat);
 skyrme_status on_current_device(const void *const *ptrs, int n);
 
 // Kernels (asynchronous, return the launch error)
+// One step on the tile kernel: FP64 gradient flows, FP32 without a tensor-map encoder
 cudaError_t launch_step(const skyrme_lattice &lat, const FlowArgs &a, cudaStream_t s);
 // The FP64 step (flow_f64.cu; not for the gradient flow); a whole lattice in
 // ARRESTED mode corrects its own mispredicted decisions inside it.
