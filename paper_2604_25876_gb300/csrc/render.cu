@@ -219,7 +219,6 @@ struct RayParams {
     float viewf[9], aspectf, halff[3], sf, boxf[3], eyef[3];
     float miss;         // every channel of a pixel without a sample
     double levelset, scale, brightness, step;
-    int skip;           // samples below the level set may be passed over without FP64
     int threshold_key;  // density_key of a value just below the level set
     float threshold;    // the same value, rounded down
     BrickLevels bricks;
@@ -371,14 +370,59 @@ __device__ __forceinline__ float pixel_value(double sum, double brightness)
     return (float)v;
 }
 
+// Whether the ray of pixel (ix, iy) may have a sample that counts: it meets the
+// box, and a coarse brick near the level set.  FP32, along the unnormalised ray
+// o + t d.  The box is widened by 1e-4, a hundred times the rounding of a point
+// on the ray there; the bricks cover a cell more than their sites, against the
+// rounding and the quarter cell that each crossing goes on past the face.  The
+// LANES lanes of `group` look at an equal part of the ray each (sub: which).
+template <int LANES>
+__device__ __forceinline__ bool ray_may_count(const RayParams &rp, int ix, int iy, int sub, unsigned group)
+{
+    const float u = (2.0f * ((float)ix + 0.5f) / (float)rp.width - 1.0f) * rp.aspectf;
+    const float v = 2.0f * ((float)iy + 0.5f) / (float)rp.height - 1.0f;
+    float d[3], tn = 0.0f, tf = 1e30f;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        d[i] = rp.viewf[3 * i] * u + rp.viewf[3 * i + 1] * v - rp.viewf[3 * i + 2] * (float)kRenderFocal;
+        const float b = rp.boxf[i] + 1e-4f, id = 1.0f / d[i];
+        const float t0 = (-b - rp.eyef[i]) * id, t1 = (b - rp.eyef[i]) * id;
+        tn = fmaxf(tn, fminf(t0, t1));  // fmin, fmax pass over NaN
+        tf = fminf(tf, fmaxf(t0, t1));
+    }
+    if (!(tn <= tf) || !rp.bricks.coarse.bits) return tn <= tf;
+    const float quarter = 0.25f / (rp.sf * sqrtf(u * u + v * v + (float)(kRenderFocal * kRenderFocal)));
+    float gd[3], igd[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) gd[a] = d[a] * rp.sf, igd[a] = fabsf(1.0f / gd[a]);
+    const float part = (tf - tn) * (1.0f / LANES), end = sub == LANES - 1 ? tf : tn + part * (float)(sub + 1);
+    bool hit = false;
+    for (float t = tn + part * (float)sub; t <= end;) {
+        float g[3], e;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) g[a] = fmaf(t, gd[a], rp.eyef[a] * rp.sf + rp.halff[a]);
+        if (!empty_brick(rp.bricks.coarse, g, gd, igd, e)) {
+            hit = true;
+            break;
+        }
+        t += fmaxf(e, 0.0f) + quarter;
+    }
+    return LANES == 1 ? hit : __any_sync(group, hit) != 0;
+}
+
 // The plain march, one ray per thread (8 x 4 pixels per warp): where no sample
-// can be passed over (a level set or scale that is not positive).
+// can be passed over (a level set or scale that is not positive), and where a
+// ray takes so few that the search costs more (few_samples).
 __global__ void __launch_bounds__(32) k_render_rays_plain(const __grid_constant__ RayParams rp,
                                                           const dvec4 *__restrict__ vol, float4 *rgba)
 {
     const int tiles_x = (rp.width + 7) >> 3, ty0 = blockIdx.x / tiles_x, tx0 = blockIdx.x - ty0 * tiles_x;
     const int ix = 8 * tx0 + (threadIdx.x & 7), iy = 4 * ty0 + (threadIdx.x >> 3);
     if (ix >= rp.width || iy >= rp.height) return;
+    if (!ray_may_count<1>(rp, ix, iy, 0, 0u)) {
+        rgba[(size_t)iy * rp.width + ix] = make_float4(rp.miss, rp.miss, rp.miss, rp.miss);
+        return;
+    }
     double d[3], tnear, tfar, sum[4] = {0.0, 0.0, 0.0, 0.0};
     pixel_ray(rp, ix, iy, d, tnear, tfar);
     int k = 0;
@@ -430,47 +474,9 @@ __global__ void __launch_bounds__(128) k_render_rays(const __grid_constant__ Ray
     const int ix = 4 * tx0 + 2 * (warp & 1) + ((lane >> 3) & 1), iy = 4 * ty0 + 2 * (warp >> 1) + (lane >> 4);
     if (ix >= rp.width || iy >= rp.height) return;  // whole groups
     float *out = reinterpret_cast<float *>(rgba + ((size_t)iy * rp.width + ix));
-    {
-        // Pixels whose ray misses the box, or meets no brick near the level
-        // set: FP32, along the unnormalised ray o + t d.  The box is widened
-        // by 1e-4, a hundred times the rounding of a point on the ray there;
-        // the bricks cover a cell more than their sites, against the rounding
-        // and the quarter cell that each crossing goes on past the face.
-        const float u = (2.0f * ((float)ix + 0.5f) / (float)rp.width - 1.0f) * rp.aspectf;
-        const float v = 2.0f * ((float)iy + 0.5f) / (float)rp.height - 1.0f;
-        float d[3], tn = 0.0f, tf = 1e30f;
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            d[i] = rp.viewf[3 * i] * u + rp.viewf[3 * i + 1] * v - rp.viewf[3 * i + 2] * (float)kRenderFocal;
-            const float b = rp.boxf[i] + 1e-4f, id = 1.0f / d[i];
-            const float t0 = (-b - rp.eyef[i]) * id, t1 = (b - rp.eyef[i]) * id;
-            tn = fmaxf(tn, fminf(t0, t1));  // fmin, fmax pass over NaN
-            tf = fminf(tf, fmaxf(t0, t1));
-        }
-        bool any = tn <= tf;
-        if (any && rp.bricks.coarse.bits) {
-            const float quarter = 0.25f / (rp.sf * sqrtf(u * u + v * v + (float)(kRenderFocal * kRenderFocal)));
-            float gd[3], igd[3];
-#pragma unroll
-            for (int a = 0; a < 3; ++a) gd[a] = d[a] * rp.sf, igd[a] = fabsf(1.0f / gd[a]);
-            const float part = (tf - tn) * 0.125f, end = sub == 7 ? tf : tn + part * (float)(sub + 1);
-            bool hit = false;
-            for (float t = tn + part * (float)sub; t <= end;) {
-                float g[3], e;
-#pragma unroll
-                for (int a = 0; a < 3; ++a) g[a] = fmaf(t, gd[a], rp.eyef[a] * rp.sf + rp.halff[a]);
-                if (!empty_brick(rp.bricks.coarse, g, gd, igd, e)) {
-                    hit = true;
-                    break;
-                }
-                t += fmaxf(e, 0.0f) + quarter;
-            }
-            any = __any_sync(group, hit);
-        }
-        if (!any) {
-            if (sub < 4) out[sub] = rp.miss;
-            return;
-        }
+    if (!ray_may_count<8>(rp, ix, iy, sub, group)) {
+        if (sub < 4) out[sub] = rp.miss;
+        return;
     }
     double d[3], tnear, tfar;
     pixel_ray(rp, ix, iy, d, tnear, tfar);
@@ -609,6 +615,29 @@ static bool render_threshold(const skyrme_render_params &p, double *value, int *
     return true;
 }
 
+// Whether the rays take so few samples that the plain march is the faster one.
+// The search sets a ray up in FP64 in eight lanes, which costs a picture that
+// fills the chip as much as 25 samples of the march, and 45 where nearly every
+// sample counts (a low level set); a march of few rays does not fill it.  Judged
+// by the ray through the picture's centre and the pixels that the box covers.
+// Search and plain march, us, 1024 x 768 pixels of a 40^3 volume, level set 0.2:
+// 5.4 samples 964 and 208, 11 967 and 296, 23 977 and 495, 45 992 and 870, 91 1016
+// and 1641 (a whole render's bricks help the search: 45 samples 1.2 times faster);
+// 320 x 240 pixels of 400 x 12 x 400 edge on, 8 samples: 27 and 44.
+static bool few_samples(const RayParams &rp)
+{
+    double chord = 1e300, area = 0.0;  // of the box; the area as seen
+    for (int i = 0; i < 3; ++i) {
+        const double d = fabs(rp.view[3 * i + 2]);
+        if (d > 0.0) chord = std::min(chord, 2.0 * rp.box[i] / d);
+        area += 4.0 * rp.box[(i + 1) % 3] * rp.box[(i + 2) % 3] * d;
+    }
+    // a picture is 2 eye / focal high where the box is
+    const double high = rp.height * (kRenderFocal / (2.0 * kRenderEye));
+    const double hits = std::min(area * high * high, (double)rp.width * rp.height);
+    return chord < rp.step * std::min(rp.levelset < 0.01 ? 48.0 : 24.0, 0.1 * sqrt(hits));
+}
+
 // Brick tables of a whole render in `bytes` of scratch: the smallest fine
 // bricks whose bits fit in 32 KiB (a ray's lookups find them in L1), coarse
 // ones four times as wide.  Returns the bytes used (0: none).
@@ -698,12 +727,12 @@ static cudaError_t ray_kernel(const int n[3], const void *vol, const skyrme_rend
     rp.miss = (float)(0.0 * p.brightness);
     double threshold = 0.0;
     rp.threshold_key = 0;
-    rp.skip = render_threshold(p, &threshold, &rp.threshold_key) ? 1 : 0;
+    const bool skip = render_threshold(p, &threshold, &rp.threshold_key);
     rp.threshold = (float)(threshold * (1.0 - 1e-6));
     rp.bricks = br;
     float4 *out = reinterpret_cast<float4 *>(rgba);
     const dvec4 *v = static_cast<const dvec4 *>(vol);
-    if (rp.skip) {
+    if (skip && !few_samples(rp)) {
         const long long tiles = (long long)((p.width + 3) / 4) * ((p.height + 3) / 4);
         k_render_rays<<<(unsigned)tiles, 128, 0, s>>>(rp, v, out);
     } else {

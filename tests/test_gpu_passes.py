@@ -114,6 +114,28 @@ def test_whole_render_equals_the_plain_march_bit_for_bit(n, view, levelset, scal
     assert np.array_equal(img.cpu().numpy(), ref)
 
 
+# rays of a few samples and of none, which the plain march takes behind the same
+# tests of the box and the bricks: coarse steps, thin boxes face on and edge on,
+# pictures of few and many pixels on either side of the choice
+@pytest.mark.parametrize("n,view", [((33, 32, 35), None), ((33, 32, 35), 2), ((6, 90, 80), 1), ((6, 90, 80), None),
+                                    ((80, 90, 6), None), ((5, 5, 5), 1)])
+@pytest.mark.parametrize("levelset,scale,step", [(0.2, 4.0, 1.0), (0.2, 4.0, 0.2), (0.2, 4.0, 0.07), (1e-4, 4.0, 0.05),
+                                                 (0.9, 30.0, 0.12), (0.0, 1.0, 0.5), (0.05, 4.0, 0.03)])
+@pytest.mark.parametrize("width,height", [(13, 9), (400, 300)])
+def test_rays_of_few_samples_equal_the_plain_march_bit_for_bit(n, view, levelset, scale, step, width, height):
+    h = 0.25
+    lat, st, _ = on_gpu(field(n, h, 4), h, 64)
+    p = dict(width=width, height=height, view=None if view is None else rotation(view),
+             levelset=levelset, transfer_scale=scale, step=step)
+    for bright in (1.0, -2.0):
+        p["brightness"] = bright
+        img = sk.render(lat, st, sk.render_params(**p))
+        vol = sk.render_volume(lat, st)
+        assert torch.equal(img, sk.render_rays(vol, sk.render_params(**p)))
+        ref = oracle.render_volume(vol.cpu().numpy(), **p).astype(np.float32)
+        assert np.array_equal(img.cpu().numpy().view(np.int32), ref.view(np.int32))
+
+
 def test_rays_pass_over_no_sample_that_is_not_finite():
     """Infinite and NaN densities count as the plain march counts them."""
     rng = np.random.default_rng(2)
