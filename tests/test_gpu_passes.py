@@ -192,6 +192,25 @@ def test_product_seed_matches_oracle(n, h, K, scale, prec, sym):
     assert sk.read_report(lat, st)["steps"] == 0
 
 
+# sites taken 256 at a time across rows and planes: planes smaller than that,
+# a last block of few sites, a single block
+@pytest.mark.parametrize("n", [(5, 5, 5), (37, 6, 7), (300, 6, 6), (6, 5, 400)])
+@pytest.mark.parametrize("prec", [64, 32])
+def test_product_seed_of_thin_lattices_matches_oracle(n, prec):
+    h, K = 0.25, 3
+    rng = np.random.default_rng(1)
+    pos, q = rng.uniform(-0.5, 0.5, size=(K, 3)), rng.normal(size=(K, 4))
+    q /= np.linalg.norm(q, axis=1, keepdims=True)
+    lat = sk.Lattice(n, h, 1.0, prec)
+    st = sk.State(lat, DEV)
+    st.phi.fill_(3.0)
+    st.vel.fill_(3.0)
+    sk.init_field(lat, sk.Seed.product(pos, q, 1.0, True), st)
+    ref = oracle.seed_product(n, h, pos, q, 1.0, True)
+    assert np.max(np.abs(st.phi[0].double().cpu().numpy() - ref)) <= (1e-12 if prec == 64 else 1.2e-7)
+    assert torch.equal(st.phi[0], st.phi[1]) and not st.vel.any().item()
+
+
 # positions so far off that r^2 overflows (such a constituent is the vacuum),
 # scales whose reciprocal overflows or is 0, and scales at the ends of the
 # table's range; on both sides of the sizes from which the table and the
