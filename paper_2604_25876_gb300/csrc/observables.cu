@@ -42,6 +42,8 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
+
 #include "lattice_sites.cuh"
 #include "skyrme_device.cuh"
 #include "skyrme_internal.h"
@@ -51,7 +53,7 @@ namespace skyrme {
 constexpr int kObsCtas = 152;
 constexpr int kObsThreads = 256;
 constexpr int kObsSums = 32;   // doubles per record
-constexpr int kObsPlanes = 4;  // x-planes of a work item (y, z and their products stay put)
+constexpr int kObsPlanes = 4;  // x-planes of a thread's run (y, z and their products stay put)
 
 // record layout
 enum {
@@ -68,6 +70,7 @@ template <typename T> struct ObsArgs {
     double *parts;
     int n0, n1, n2;
     int blocks, items;  // (y, z) blocks of 256 sites, work items
+    int share;          // runs of planes that share an item where a plane's sites fit in a block
     double h, two_m2;
     double K144, k1sq, k1qu;  // 144 h^2, and 1/(12h) to the 2nd and 4th power
 };
@@ -108,9 +111,10 @@ __global__ void __launch_bounds__(kObsThreads) k_observables(const __grid_consta
     for (int q = 0; q < kObsSums; ++q) acc[q] = 0.0;
 
     for (int it = blockIdx.x; it < a.items; it += gridDim.x) {
-        const int xc = it / a.blocks;
-        const int s = (it - xc * a.blocks) * kObsThreads + threadIdx.x;
-        if (s >= iy * iz) continue;
+        const int xi = it / a.blocks, sub = a.share > 1 ? (int)threadIdx.x / (iy * iz) : 0;
+        const int xc = xi * a.share + sub;
+        const int s = (it - xi * a.blocks) * kObsThreads + (int)threadIdx.x - sub * iy * iz;
+        if (sub >= a.share || s >= iy * iz) continue;
         const int y = 2 + s / iz, z = 2 + s % iz;
         const double r1 = ((double)y - 0.5 * (a.n1 - 1)) * a.h - X[1];
         const double r2 = ((double)z - 0.5 * (a.n2 - 1)) * a.h - X[2];
@@ -262,7 +266,13 @@ static skyrme_status observables_impl(const skyrme_lattice &lat, const FlowArgs 
     a.n1 = lat.n[1];
     a.n2 = lat.n[2];
     a.blocks = ((a.n1 - 4) * (a.n2 - 4) + kObsThreads - 1) / kObsThreads;
-    a.items = a.blocks * ((a.n0 - 4 + kObsPlanes - 1) / kObsPlanes);
+    // Small planes: items of several runs, where one run each would be more items than
+    // CTAs (3000 x 6 x 7 FP32 370 us so, 118 now); no more to an item than that
+    // takes, for a CTA's warps share its SM's FP64 pipe (400 x 10 x 10 110 us with one
+    // each, 156 with blocks filled).
+    const int runs = (a.n0 - 4 + kObsPlanes - 1) / kObsPlanes;
+    a.share = std::max(1, std::min(kObsThreads / ((a.n1 - 4) * (a.n2 - 4)), (runs + kObsCtas - 1) / kObsCtas));
+    a.items = a.blocks * ((runs + a.share - 1) / a.share);
     a.h = lat.h;
     // the derivatives are carried without their 1/(12h) = k1 (d_k phi = k1 u_k):
     // Y, A, B, H, Z then hold powers 1, 2, 2, 3, 4 of 12h, taken out of the sums

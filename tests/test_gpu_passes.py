@@ -86,6 +86,21 @@ def test_observables_match_oracle_at_the_edges_of_the_work_split(n, prec):
     assert g["D"] == pytest.approx(o["D"], abs=tol * o["E"] * max(1.0, np.max(np.abs(o["V"]))))
 
 
+# planes of so few sites that several runs along x share a block: one, some and
+# many to a block, the last block's only partly there, one plane a run
+# (a field cut so short that its mean square radius is negative has no R)
+@pytest.mark.parametrize("n", [(6, 6, 6), (9, 6, 7), (61, 8, 9), (300, 6, 6), (300, 6, 7), (45, 12, 20), (30, 16, 15), (1300, 7, 8), (700, 20, 9),
+                               (1217, 6, 7)])
+@pytest.mark.parametrize("prec", [64, 32])
+def test_observables_of_thin_lattices_match_oracle(n, prec):
+    lat, st, phi = on_gpu(field(n, 0.25, 1), 0.25, prec)
+    if np.isnan(oracle.observables(phi, 0.25, 1.0)["R"]):
+        with pytest.raises(sk.SkyrmeError, match="non-finite"):
+            sk.observables(lat, st)
+        return
+    test_observables_match_oracle_at_the_edges_of_the_work_split(n, prec)
+
+
 def rotation(seed):
     q = np.random.default_rng(seed).normal(size=4)
     a, b, c, d = q / np.linalg.norm(q)
