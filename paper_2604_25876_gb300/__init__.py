@@ -335,15 +335,6 @@ class Seed:
         return s, (pos, q)  # keep host arrays alive during the call
 
 
-def _pair(buf) -> _VoidP2:
-    """The addresses of buf[0] and buf[1]: in a tensor of two buffers the second
-    lies one stride behind the first (indexing would make a tensor)."""
-    if isinstance(buf, _torch().Tensor) and buf.shape[0] > 1:
-        p = buf.data_ptr()
-        return _VoidP2(p, p + buf.stride()[0] * buf.itemsize)
-    return _VoidP2(buf[0].data_ptr(), buf[1].data_ptr())
-
-
 class State:
     """Device buffers of one lattice: two field and two velocity buffers
     (torch tensors of shape (2, Nx, Ny, Nz, 4)) and the scratch block."""
@@ -358,8 +349,18 @@ class State:
         self.scratch = torch.zeros(lat.scratch_bytes(), dtype=torch.uint8, device=self.device)
 
     def c(self) -> c_state:
-        scratch = self.scratch
-        return c_state(_pair(self.phi), _pair(self.vel), scratch.data_ptr(), scratch.numel())
+        # of a tensor of two buffers the second lies one stride behind the first
+        # (indexing would make a tensor)
+        phi, vel, scratch = self.phi, self.vel, self.scratch
+        tensor = _torch().Tensor
+        if isinstance(phi, tensor) and isinstance(vel, tensor) and phi.shape[0] > 1 < vel.shape[0]:
+            p, v = phi.data_ptr(), vel.data_ptr()
+            return c_state(_VoidP2(p, p + phi.stride()[0] * phi.itemsize),
+                           _VoidP2(v, v + vel.stride()[0] * vel.itemsize),
+                           scratch.data_ptr(), scratch.numel())
+        return c_state(_VoidP2(phi[0].data_ptr(), phi[1].data_ptr()),
+                       _VoidP2(vel[0].data_ptr(), vel[1].data_ptr()),
+                       scratch.data_ptr(), scratch.numel())
 
     def report(self, stream=None) -> dict:
         return read_report(self.lat, self, stream)
@@ -387,7 +388,7 @@ def init_field(lat: Lattice, seed: Seed, st: State, stream=None):
     del keep
 
 
-def _loadable(lat: Lattice, st: State, cs: c_state, t) -> bool:
+def _loadable(lat: Lattice, st: State, t) -> bool:
     """Whether the load kernel can read the tensor where it is: a plain
     contiguous tensor of the state's device, precision and shape, aligned to a
     site and apart from the state's buffers."""
@@ -398,13 +399,15 @@ def _loadable(lat: Lattice, st: State, cs: c_state, t) -> bool:
             t.dtype != lat.dtype or t.shape != st.phi.shape[1:] or not t.is_contiguous() or \
             t.requires_grad or t.is_neg() or t.numel() == 0:
         return False
-    site, size, a = 4 * t.element_size(), t.numel() * t.element_size(), t.data_ptr()
-    if a < cs.scratch + cs.scratch_bytes and cs.scratch < a + size:
+    item, a = t.itemsize, t.data_ptr()
+    size = t.numel() * item
+    b = a + size
+    # (from a pair's first buffer to the end of its second)
+    p, v, s = st.phi.data_ptr(), st.vel.data_ptr(), st.scratch.data_ptr()
+    if a < p + st.phi.stride()[0] * item + size and p < b or a < v + st.vel.stride()[0] * item + size and v < b or \
+            a < s + st.scratch.numel() and s < b:
         return False
-    for p in (cs.phi[0], cs.phi[1], cs.vel[0], cs.vel[1]):
-        if a < p + size and p < a + size:
-            return False
-    return a % site == 0
+    return a % (4 * item) == 0
 
 
 def load_field(lat: Lattice, st: State, phi, stream=None):
@@ -413,7 +416,7 @@ def load_field(lat: Lattice, st: State, phi, stream=None):
     torch = _torch()
     t = torch.as_tensor(np.asarray(phi) if not isinstance(phi, torch.Tensor) else phi)
     cl, cs = lat.c(), st.c()
-    if stream is None and _loadable(lat, st, cs, t):
+    if stream is None and _loadable(lat, st, t):
         # read by the load kernel itself, on the current stream as the copy is
         _check(_on(st.device).skyrme_load_field_from(ctypes.byref(cl), ctypes.byref(cs),
                                                      ctypes.c_void_p(t.data_ptr()),
