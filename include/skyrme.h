@@ -161,6 +161,13 @@ skyrme_status skyrme_load_field_from(const skyrme_lattice *lat, skyrme_state *st
  * at interior sites.  `report` (nullable, host) receives the latest
  * iteration's results, which synchronises the stream.  Returns
  * SKYRME_ENONFINITE (sticky) once a non-finite value has appeared.
+ * Flows of different states may run on different streams at the same time,
+ * but ARRESTED flows of FP32 lattices should not: their launches wait inside
+ * for the decision, and start while the launch before them still ends, so two
+ * of them could each hold some SMs and wait for the rest of themselves; the
+ * waits then end after 2 s with SKYRME_ETIMEOUT.  Use skyrme_batch for several
+ * lattices at once, or one stream.  (FP64 launches that wait are cooperative
+ * and do not overlap their predecessors.)
  * From 256 iterations on, on a stream that is not being captured, the call
  * captures 128 iterations into a CUDA graph on a stream of its own and
  * replays it on `stream` (fewer GPU cycles per launch); the graph and that

@@ -418,14 +418,16 @@ def test_fp64_steps_in_a_launch_are_capped(n, steps, launches, mode):
     assert bench.step_launches(wl, 64, steps) == launches
 
 
-# launches that wait inside (for the arrest decision, for the next step) on two
-# streams at a time: one or two CTAs to an SM, some SMs idle, different lattices
+# Two flows on two streams at a time: FP64 launches that wait inside (for the
+# arrest decision, for the next step), with one or two CTAs to an SM, some SMs
+# idle, different lattices; and the modes whose launches do not wait.
 @pytest.mark.parametrize("na,nb", [((48, 48, 48), (48, 48, 48)), ((20, 22, 24), (70, 66, 68)),
                                    ((70, 66, 68), (66, 70, 64))])
-@pytest.mark.parametrize("mode,dt", [(sk.ARRESTED, 0.03), (sk.NEWTON, 0.004)])
-def test_two_fp64_flows_on_two_streams_equal_the_flows_alone(na, nb, mode, dt):
+@pytest.mark.parametrize("prec,mode,dt", [(64, sk.ARRESTED, 0.03), (64, sk.NEWTON, 0.004), (64, sk.GRADIENT, 1e-5),
+                                          (32, sk.NEWTON, 0.004), (32, sk.GRADIENT, 1e-5)])
+def test_two_flows_on_two_streams_equal_the_flows_alone(na, nb, prec, mode, dt):
     h, steps, launches = 0.25, 40, 4
-    pairs = [[on_gpu(field(n, h, 2 + k), h, 64)[:2] for k, n in enumerate((na, nb))] for _ in range(2)]
+    pairs = [[on_gpu(field(n, h, 2 + k), h, prec)[:2] for k, n in enumerate((na, nb))] for _ in range(2)]
     for lat, st in pairs[0]:
         for _ in range(launches):
             sk.flow_step(lat, dt, steps, mode, st)
