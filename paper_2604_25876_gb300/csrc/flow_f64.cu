@@ -30,8 +30,8 @@
 //  * A launch runs several steps of a small lattice (kLaunchSites, kLaunchSteps): every CTA
 //    waits for the decision and goes on to the next step, over one more barrier
 //    when sites were corrected.  One step per launch and now, us per step in a
-//    graph and on a stream: 24 x 26 x 28 26.9 and 29.2 -> 25.7 and 26.0, 48^3
-//    73.7 and 76.3 -> 72.5 and 73.0, 90 x 75 x 83 326 and 329 -> 325 and 325.
+//    graph and on a stream: 24 x 26 x 28 26.9 and 29.2 -> 25.1 and 25.2, 48^3
+//    73.7 and 76.3 -> 72.1 and 72.2, 90 x 75 x 83 326 and 329 -> 325 and 326.
 //  * Launches whose CTAs wait for one another (for the decision, or for the next
 //    step) are cooperative: the CTAs of one are resident together, whatever other
 //    streams run.  Consecutive launches are not programmatic dependents, whose
@@ -39,9 +39,9 @@
 //    could then each hold some SMs and wait for CTAs that the other leaves no
 //    room for.
 //  * Measured (us per iteration, tile kernel and fix-up launch before -> now):
-//    48^3 103.6 -> 73, 64^3 187 -> 153, 128^3 1392 -> 1166 (1.63 G
-//    site-updates/s, 334 instructions per site at the measured FP64 FMA rate),
-//    90 x 75 x 83 lightly bound 409 -> 326, 72 x 80 x 100 sextic 520 -> 429.
+//    48^3 103.6 -> 72, 64^3 187 -> 153, 128^3 1392 -> 1166 (1.635 G
+//    site-updates/s, 322 instructions per site at the measured FP64 FMA rate: full),
+//    90 x 75 x 83 lightly bound 409 -> 325, 72 x 80 x 100 sextic 520 -> 417.
 //  * The arrest decision falls in the last CTA to finish; the launch is
 //    cooperative, and every warp corrects its own sites when the decision that
 //    the step ran with was wrong (flow_generic.cu has the scheme).

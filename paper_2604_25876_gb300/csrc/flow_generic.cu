@@ -661,7 +661,7 @@ cudaError_t launch_step(const skyrme_lattice &lat, const FlowArgs &a, cudaStream
     // steps the other modes take, and then multiplies a rounding difference by
     // up to 10^9 in 20 steps (a fifth of a sample of 40 FP64 gradient flows): FP64
     // fields keep the tile kernel and its roundings in that mode.  It would gain
-    // what the other modes do (48^3 92 -> 73 us a step), which run on flow_f64.cu
+    // what the other modes do (48^3 92 -> 72 us a step), which run on flow_f64.cu
     // and do not come here.
     if (lat.precision == 64)
         return launch_tile<double, 0>(lat, make_params<double>(a, a.step_parts), nullptr, nullptr, s);
