@@ -401,7 +401,9 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_step_f64(const __grid_con
 #pragma unroll
                     for (int i = 0; i < 4; ++i) acc[i] += dens[i];
                     acc[4] += f2;
-                    mx = max(mx, __double_as_longlong(f2));  // (f2 >= 0: ordered as its bits)
+                    // (f2 >= 0: ordered as its bits; NaN, above infinity's, is passed over)
+                    const long long fb = __double_as_longlong(f2);
+                    if (fb <= 0x7ff0000000000000LL) mx = max(mx, fb);
                     if constexpr (EXT) acc[6] += dens[4];
                 }
             }

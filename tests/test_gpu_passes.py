@@ -283,6 +283,23 @@ def test_large_fp32_product_seed_is_the_rounded_fp64_seed(n, h, K, scale, sym):
     assert torch.all((phi[32] - ref).abs()[off] <= 1.3e-7 * ref.abs()[off])
 
 
+# where the force is NaN at some sites, delta is the largest of the others' (every
+# lane, warp and CTA keeps its own), as the oracle's comparison passes over NaN
+@pytest.mark.parametrize("n", [(12, 13, 14), (24, 26, 28)])
+@pytest.mark.parametrize("prec,tol", [(64, 1e-10), (32, 1e-4)])
+def test_delta_passes_over_sites_that_are_not_finite(n, prec, tol):
+    h = 0.25
+    phi = oracle.seed_rational_map(n, h, 2, 0.7)
+    phi[n[0] // 2 - 1, n[1] // 2, n[2] // 2, 1] = np.nan  # among the strongest forces
+    lat, st, phi = on_gpu(phi, h, prec)
+    with pytest.raises(sk.SkyrmeError, match="non-finite"):
+        sk.flow_step(lat, 1e-3, 1, sk.NEWTON, st)
+    rep = sk.read_report(lat, st)
+    _, f, _ = oracle.forces(phi, h, 1.0)
+    ref = np.nanmax(np.linalg.norm(f, axis=-1))
+    assert rep["delta"] == pytest.approx(ref, rel=tol) and np.isnan(rep["E"])
+
+
 def captured_nodes(call):
     """How many kernels, copies and memsets ``call`` puts on its stream."""
     cu = ctypes.CDLL("libcuda.so.1")
