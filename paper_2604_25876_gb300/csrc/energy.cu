@@ -232,7 +232,8 @@ __device__ __forceinline__ void finish_energy(Ctrl *c, double *parts, const doub
             r += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
         }
         r = warp_sum(r);
-        if (lane == 0) buf[warp] = scale[warp] * r;
+        // (no sextic term: 0, also where the sum of the squares overflows)
+        if (lane == 0) buf[warp] = warp == 4 && scale[4] == 0.0 ? 0.0 : scale[warp] * r;
     }
     __syncthreads();
     if (tid == 0) {

@@ -66,6 +66,21 @@ def test_energy_matches_oracle_at_the_edges_of_the_work_split(n, prec, tol, mode
     assert sk.energy(lat, st) == eg  # the same order every time
 
 
+# potentials without the sextic term take the extended pass, whose sextic sum may
+# overflow in FP32 on a field that is far from normalised: it counts for nothing
+@pytest.mark.parametrize("model", [{"m_w": 1.0}, {"m_y": 0.3, "m_z": 0.2}])
+def test_energy_without_the_sextic_term_does_not_overflow_with_it(model):
+    n, h = (12, 13, 14), 0.25
+    lat, st, phi = on_gpu(1e6 * field(n, h), h, 32, **model)
+    om = oracle.Model(1.0, *(model.get(k, 0.0) for k in ("m_y", "m_z", "m_w", "c6")))
+    eo, eg = oracle.energy(phi, h, om), sk.energy(lat, st)
+    assert np.isfinite(list(eg.values())).all()
+    # (E4 is a difference of terms of its size; E0 in FP32 takes 1 - phi^0 from the
+    # pions of a unit field, so it is not the oracle's here)
+    assert eg["E2"] == pytest.approx(eo["E2"], rel=2e-5)
+    assert eg["E"] == pytest.approx(eg["E2"] + eg["E4"] + eg["E0"], rel=1e-12)
+
+
 # (a lattice one site wide along an axis has no charge, so no observables)
 @pytest.mark.parametrize("n", [(6, 7, 21), (9, 20, 37), (7, 21, 20), (70, 13, 8), (12, 40, 53),
                                (8, 9, 300)])
