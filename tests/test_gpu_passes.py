@@ -552,17 +552,25 @@ def test_load_field_gives_the_same_state_from_every_source(n, prec):
         assert not st.vel.any().item()
         rep = sk.read_report(lat, st)
         assert rep["steps"] == 0 and rep["cur"] == 0 and rep["status"] == 0
+    with pytest.raises(RuntimeError):  # shapes that do not broadcast stay refused
+        sk.load_field(lat, sk.State(lat, DEV), t[1:])
+
+
+@pytest.mark.parametrize("n", [(5, 5, 5), (12, 40, 53)])
+@pytest.mark.parametrize("prec", [64, 32])
+def test_load_field_into_buffers_apart(n, prec):
+    lat = sk.Lattice(n, 0.25, 1.0, prec)
+    t = torch.from_numpy(field(n, 0.25, 3)).to(DEV, lat.dtype)
+    ref = torch.from_numpy(oracle.apply_vacuum_boundary(t.double().cpu().numpy())).to(DEV, lat.dtype)
     st, wide = sk.State(lat, DEV), torch.zeros((4,) + t.shape, dtype=lat.dtype, device=DEV)
-    st.phi = wide[::2]  # buffers apart, the source the second of them
+    st.phi = wide[::2]  # the source is the second of them
     wide[2].copy_(t)
     sk.load_field(lat, st, wide[2])
     assert torch.equal(wide[0], ref) and torch.equal(wide[2], ref) and not wide[1::2].any().item()
-    st = sk.State(lat, DEV)  # buffers of their own
+    st = sk.State(lat, DEV)  # tensors of their own
     st.phi, st.vel = [torch.empty_like(t) for _ in range(2)], [torch.empty_like(t) for _ in range(2)]
     sk.load_field(lat, st, t)
     assert torch.equal(st.phi[0], ref) and torch.equal(st.phi[1], ref)
-    with pytest.raises(RuntimeError):  # shapes that do not broadcast stay refused
-        sk.load_field(lat, sk.State(lat, DEV), t[1:])
 
 
 def test_load_field_from_rejects_null_misaligned_and_overlapping_sources():
